@@ -68,8 +68,10 @@ typedef enum {
 
 /* Execution paths.  PLAIN_FP32: one kernel launch per sub-step (observe,
  * each policy layer, sample, env step) per step, FP32 SIMT, launched from the
- * host every step.  BATCHED_FP32: the same kernels, captured as a CUDA graph
- * per chunk of steps.  BATCHED_BF16: policy GEMMs (and the landscape
+ * host every step.  BATCHED_FP32: the same arithmetic, captured as a CUDA graph
+ * per chunk of steps; for the control env and the acrobot with hidden widths up
+ * to 256 one fused kernel runs a whole chunk (equal records, byte for byte).
+ * BATCHED_BF16: policy GEMMs (and the landscape
  * cross-term) on the tcgen05 tensor cores in BF16 with FP32 accumulation;
  * for the control env, the economy with 16-128-128-20 / -10 policies and at
  * most 384 agents per env, and the landscape with D in {8, 16, 24} and

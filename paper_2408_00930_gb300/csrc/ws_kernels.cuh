@@ -150,6 +150,11 @@ bool control_cc_tile_ok(const PolicyShape &shape, int envs_per_cta, int threads_
 cudaError_t launch_control_cc(const Dev &d, uint32_t n_steps, int envs_per_cta, int threads_per_env,
                               cudaStream_t st);
 
+// ---- fused FP32 control path (ws_control_f32.cu) ----------------------------
+// Steps [k + off, k + off + n_steps) of every env in one launch.
+bool control_f32_supported(const PolicyShape &shape);
+cudaError_t launch_control_f32(const Dev &d, uint32_t off, uint32_t n_steps, cudaStream_t st);
+
 }  // namespace ws
 
 namespace ws {

@@ -474,6 +474,13 @@ void drop_graphs(ws_ctx *c) {
 // Paths whose chunks run as one persistent kernel launch each.
 bool fused(const ws_ctx *c) { return use_tc_control(&c->cfg) || c->L.econ_fused || c->L.land_fused; }
 
+// The classic-control envs on the batched FP32 path, for the policy widths its
+// fused kernel holds.
+bool fused_f32_control(const ws_ctx *c) {
+  return (c->cfg.env == WS_ENV_CONTROL || c->cfg.env == WS_ENV_ACROBOT) &&
+         c->cfg.path == WS_PATH_BATCHED_FP32 && control_f32_supported(c->L.pol);
+}
+
 uint32_t chunk_of(const ws_ctx *c) { return c->lc.chunk_steps; }
 
 int sm_count() {
@@ -568,6 +575,15 @@ ws_status enqueue_steps(ws_ctx *c, uint32_t n, cudaStream_t st) {
       launch_advance(c->d, m, st);
       done += m;
     }
+  } else if (fused_f32_control(c)) {
+    const uint32_t chunk = chunk_of(c);
+    for (uint32_t done = 0; done < n;) {
+      const uint32_t m = (n - done) < chunk ? (n - done) : chunk;
+      cudaError_t e = launch_control_f32(c->d, done, m, st);
+      if (e != cudaSuccess) return cuda_check(c, e, "control FP32 launch");
+      done += m;
+    }
+    launch_advance(c->d, n, st);
   } else {
     const Branch *br = c->br.aux ? &c->br : nullptr;
     for (uint32_t i = 0; i < n; ++i) launch_plain_step(c->d, i, st, br);
@@ -892,7 +908,7 @@ ws_status ws_rollout(ws_ctx *c, uint32_t n) {
   ws_status s = WS_OK;
   if (c->cfg.path == WS_PATH_PLAIN_FP32) {
     for (uint32_t i = 0; i < n && s == WS_OK; ++i) s = enqueue_steps(c, 1, c->stream);
-  } else if (fused(c)) {
+  } else if (fused(c) || fused_f32_control(c)) {
     cudaGraphExec_t g;
     s = graph_for(c, n, &g);
     if (s == WS_OK) s = cuda_check(c, cudaGraphLaunch(g, c->stream), "graph launch");
