@@ -101,12 +101,31 @@ struct TrainBufs {                 // per-chunk scratch in the state buffer
   float *h1, *h2, *out, *c1, *c2, *vout, *d1, *d2, *part;
   double *stats;                   // policy loss, value loss, entropy, clipped rows (sums)
   float *grad;                     // actor gradient, then the critic's
+  uint8_t *image;                  // packed W2 of actor and critic: forward, then backward operands
 };
 struct TrainGroup {  // one policy and its critic, on slots [slot0, slot0 + n_slots) of every step
   float *params, *critic;
   PolicyShape pol, crit;
   uint32_t slot0, n_slots;
 };
+// Fused forward pass of a chunk (ws_train_fwd.cu): rows [q0, q0 + rows) of a group
+// from the ring through both networks (or the critic alone) into tb's activations,
+// outputs and values, with W2 packed by launch_train_pack.
+bool train_tc_supported(const PolicyShape &p);
+bool train_fwd_has_out(int out);
+size_t train_image_bytes(const PolicyShape &p);
+void launch_train_pack(const TrainGroup &g, uint8_t *img, cudaStream_t st);
+cudaError_t launch_train_fwd(const Dev &d, const TrainGroup &g, const TrainBufs &tb, uint64_t q0,
+                             uint32_t n, uint32_t rows, int critic_only, cudaStream_t st);
+// Fused backward of the same chunk (ws_train_bwd.cu): dout (tb.out, tb.vout) through
+// both networks, the gradients added to tb.grad.  A policy without train_bwd_has_out
+// gives the gradients at the last hidden layer in tb.d1, tb.d2 and keeps the output
+// layers' weight gradients to itself.
+constexpr int kTrainMaxCtas = 160, kTrainMaxSlices = 80;
+bool train_bwd_has_out(const PolicyShape &p);
+size_t train_part_floats(const PolicyShape &p);
+cudaError_t launch_train_bwd(const Dev &d, const TrainGroup &g, const TrainBufs &tb, uint64_t q0,
+                             uint32_t n, uint32_t rows, cudaStream_t st);
 // Scratch sized for the widest policy of the context (and its critic).
 size_t train_scratch_bytes(const PolicyShape &pol);
 TrainBufs train_bufs(uint8_t *base, const PolicyShape &pol);

@@ -749,10 +749,10 @@ void hgemm(const Dev &d, dim3 g, cudaStream_t st, const float *A, int lda, const
 // Forward of one three-layer MLP for a chunk (rows x w0 row-major input),
 // keeping the tanh activations h1, h2.
 void mlp_forward(const Dev &d, const PolicyShape &sh, const float *params, const float *X, float *h1,
-                 float *h2, float *out, int rows, cudaStream_t st) {
+                 float *h2, float *out, int rows, cudaStream_t st, int first = 0) {
   const float *in[3] = {X, h1, h2};
   float *o[3] = {h1, h2, out};
-  for (int l = 0; l < 3; ++l) {
+  for (int l = first; l < 3; ++l) {
     const int K = sh.w[l], N = sh.w[l + 1];
     const float *W = params + sh.layer_offset(l), *b = W + (size_t)K * N;
     if (N <= kThin) {
@@ -787,16 +787,45 @@ void mlp_forward(const Dev &d, const PolicyShape &sh, const float *params, const
   }
 }
 
+// The fused kernels' shapes, unless the launch asks for FP32 CUDA-core GEMMs.
+bool use_train_tc(const Dev &d, const PolicyShape &p) { return !d.update_simt && train_tc_supported(p); }
+
+// Forward of a chunk (rows from q0 of the group) through the policy (unless
+// critic_only) and the critic: one fused launch where the shape allows it, else
+// layer by layer from the gathered inputs.
+void chunk_forward(const Dev &d, const TrainBufs &tb, const TrainGroup &G, uint32_t n, size_t q0,
+                   int rows, bool critic_only, cudaStream_t st) {
+  if (use_train_tc(d, G.pol) &&
+      launch_train_fwd(d, G, tb, q0, n, (uint32_t)rows, critic_only, st) == cudaSuccess) {
+    if (!critic_only && !train_fwd_has_out(G.pol.w[3]))
+      mlp_forward(d, G.pol, G.params, tb.x, tb.h1, tb.h2, tb.out, rows, st, 2);
+    return;
+  }
+  if (!critic_only) mlp_forward(d, G.pol, G.params, tb.x, tb.h1, tb.h2, tb.out, rows, st);
+  mlp_forward(d, G.crit, G.critic, tb.x, tb.c1, tb.c2, tb.vout, rows, st);
+}
+
+// Rows per chunk: whole rounds of 128-row tiles over the SMs for the fused
+// kernels, so that no round is partly filled.
+size_t chunk_rows(const Dev &d, const PolicyShape &p) {
+  if (!use_train_tc(d, p)) return kTrainChunk;
+  int dev = 0, sms = 148;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const size_t round = 128 * (size_t)sms;
+  return round <= (size_t)kTrainChunk ? kTrainChunk / round * round : kTrainChunk;
+}
+
 // Backward through one three-layer MLP for a chunk: X [rows][w0], h1, h2 the
 // tanh activations, dout [rows][w3] the gradient at the output.  Per layer the
 // weight gradient as row-slice partials (and the bias row), summed into
 // grad in slice order, then the data gradient into the layer below.
 void mlp_backward(const Dev &d, const PolicyShape &sh, const float *params, const float *X,
                   const float *h1, const float *h2, const float *dout, float *grad, float *d1, float *d2,
-                  float *part, int rows, cudaStream_t st) {
+                  float *part, int rows, cudaStream_t st, int last = 0) {
   const float *ain[3] = {X, h1, h2};
   float *dl[3] = {nullptr, d1, d2};
-  for (int l = 2; l >= 0; --l) {
+  for (int l = 2; l >= last; --l) {
     const int M = sh.w[l], N = sh.w[l + 1];
     const int sr = slice_rows(M, N), nz = (rows + sr - 1) / sr;
     const float *D = l == 2 ? dout : dl[l + 1];
@@ -833,6 +862,21 @@ void mlp_backward(const Dev &d, const PolicyShape &sh, const float *params, cons
   }
 }
 
+// Backward of a chunk through both networks, the gradients added to tb.grad.
+void chunk_backward(const Dev &d, const TrainBufs &tb, const TrainGroup &G, uint32_t n, size_t q0,
+                    int rows, cudaStream_t st) {
+  float *ga = tb.grad, *gc = tb.grad + G.pol.count();
+  if (use_train_tc(d, G.pol)) {
+    if (!train_bwd_has_out(G.pol)) {  // the output layers, down to the gradients d1 (actor), d2 (critic)
+      mlp_backward(d, G.pol, G.params, tb.x, tb.h1, tb.h2, tb.out, ga, nullptr, tb.d1, tb.part, rows, st, 2);
+      mlp_backward(d, G.crit, G.critic, tb.x, tb.c1, tb.c2, tb.vout, gc, nullptr, tb.d2, tb.part, rows, st, 2);
+    }
+    if (launch_train_bwd(d, G, tb, q0, n, (uint32_t)rows, st) == cudaSuccess) return;
+  }
+  mlp_backward(d, G.pol, G.params, tb.x, tb.h1, tb.h2, tb.out, ga, tb.d1, tb.d2, tb.part, rows, st);
+  mlp_backward(d, G.crit, G.critic, tb.x, tb.c1, tb.c2, tb.vout, gc, tb.d1, tb.d2, tb.part, rows, st);
+}
+
 // The scratch of one update chunk, carved from base (or, with base null, only
 // measured): returns its size in bytes.
 size_t train_layout(uint8_t *base, const PolicyShape &pol, TrainBufs *t) {
@@ -850,6 +894,7 @@ size_t train_layout(uint8_t *base, const PolicyShape &pol, TrainBufs *t) {
     const size_t vc = (CH + src - 1) / src * lenc;
     if (vc > part_len) part_len = vc;
   }
+  if (train_part_floats(pol) > part_len) part_len = train_part_floats(pol);
   size_t o = 0;
   auto take = [&](size_t n) {
     uint8_t *p = base ? base + o : nullptr;
@@ -873,6 +918,7 @@ size_t train_layout(uint8_t *base, const PolicyShape &pol, TrainBufs *t) {
   b.part = (float *)take(part_len * 4); // weight-gradient partials
   b.stats = (double *)take(4 * 8);
   b.grad = (float *)take((pol.count() + crit.count()) * 4);
+  b.image = take(train_image_bytes(pol));
   if (t) *t = b;
   return o;
 }
@@ -902,22 +948,20 @@ void run_update(const Dev &d, const TrainBufs &tb, const TrainGroup *groups, int
     float *ga = tb.grad, *gc = tb.grad + na;
     cudaMemsetAsync(tb.grad, 0, (na + nc) * 4, st);
     const double inv_r = 1.0 / (double)R;
-    for (size_t q0 = 0; q0 < R; q0 += kTrainChunk) {
-      const int rows = (int)((R - q0) < (size_t)kTrainChunk ? (R - q0) : (size_t)kTrainChunk);
+    const size_t CH = chunk_rows(d, G.pol);
+    if (use_train_tc(d, G.pol)) launch_train_pack(G, tb.image, st);
+    for (size_t q0 = 0; q0 < R; q0 += CH) {
+      const int rows = (int)((R - q0) < CH ? (R - q0) : CH);
       k_a2c_gather<<<nblk(rows, 256), 256, 0, st>>>(d, n, q0, (uint32_t)rows, G.slot0, G.n_slots,
                                                     G.pol.w[0], ppo ? 1 : 0, tb);
-      mlp_forward(d, G.pol, G.params, tb.x, tb.h1, tb.h2, tb.out, rows, st);
-      mlp_forward(d, G.crit, G.critic, tb.x, tb.c1, tb.c2, tb.vout, rows, st);
+      chunk_forward(d, tb, G, n, q0, rows, false, st);
       if (ppo)
         k_ppo_head<<<nblk(rows, 256), 256, 0, st>>>(d, n, q0, (uint32_t)rows, G.n_slots,
                                                     G.pol.w[3], inv_r, eps, c_v, c_e, tb);
       else
         k_a2c_head<<<nblk(rows, 256), 256, 0, st>>>(d, n, q0, (uint32_t)rows, G.n_slots,
                                                     G.pol.w[3], inv_r, c_v, c_e, tb);
-      mlp_backward(d, G.pol, G.params, tb.x, tb.h1, tb.h2, tb.out, ga, tb.d1, tb.d2, tb.part, rows,
-                   st);
-      mlp_backward(d, G.crit, G.critic, tb.x, tb.c1, tb.c2, tb.vout, gc, tb.d1, tb.d2, tb.part, rows,
-                   st);
+      chunk_backward(d, tb, G, n, q0, rows, st);
     }
     k_sgd<<<nblk(na, 256), 256, 0, st>>>(G.params, ga, na, lr);
     k_sgd<<<nblk(nc, 256), 256, 0, st>>>(G.critic, gc, nc, lr);
@@ -942,16 +986,17 @@ void launch_advantages(const Dev &d, const TrainBufs &tb, const TrainGroup *grou
                        uint32_t n, cudaStream_t st) {
   for (int gi = 0; gi < n_groups; ++gi) {
     const TrainGroup &G = groups[gi];
-    const size_t R = (size_t)n * G.n_slots;
-    for (size_t q0 = 0; q0 < R; q0 += kTrainChunk) {
-      const int rows = (int)((R - q0) < (size_t)kTrainChunk ? (R - q0) : (size_t)kTrainChunk);
+    const size_t R = (size_t)n * G.n_slots, CH = chunk_rows(d, G.pol);
+    const bool both = d.env == WS_ENV_LANDSCAPE;  // its actor rebuilds the samples
+    if (use_train_tc(d, G.pol)) launch_train_pack(G, tb.image, st);
+    for (size_t q0 = 0; q0 < R; q0 += CH) {
+      const int rows = (int)((R - q0) < CH ? (R - q0) : CH);
       k_a2c_gather<<<nblk(rows, 256), 256, 0, st>>>(d, n, q0, (uint32_t)rows, G.slot0, G.n_slots,
                                                     G.pol.w[0], 0, tb);
-      mlp_forward(d, G.crit, G.critic, tb.x, tb.c1, tb.c2, tb.vout, rows, st);
+      chunk_forward(d, tb, G, n, q0, rows, !both, st);
       k_adv_store<<<nblk(rows, 256), 256, 0, st>>>(d, n, q0, (uint32_t)rows, G.slot0, G.n_slots,
                                                    tb);
       if (d.env == WS_ENV_LANDSCAPE) {  // one group: every slot
-        mlp_forward(d, G.pol, G.params, tb.x, tb.h1, tb.h2, tb.out, rows, st);
         k_sample_store<<<nblk(rows, 256), 256, 0, st>>>(d, n, q0, (uint32_t)rows, G.n_slots, tb);
       }
     }
