@@ -95,9 +95,7 @@ void launch_returns(const Dev &d, uint32_t n_steps, cudaStream_t st);
 // ---- actor-critic updates (ws_train.cu) ---------------------------------------
 constexpr int kTrainChunk = 65536;  // rows per chunk of the update
 struct TrainBufs {                 // per-chunk scratch in the state buffer
-  float *x, *ret;
-  int32_t *act;
-  float *adv, *lpo;                // PPO: held advantage, behaviour log-probability
+  float *x;                        // observations (layer-by-layer path)
   float *h1, *h2, *out, *c1, *c2, *vout, *d1, *d2, *part;
   double *stats;                   // policy loss, value loss, entropy, clipped rows (sums)
   float *grad;                     // actor gradient, then the critic's
@@ -121,7 +119,7 @@ cudaError_t launch_train_fwd(const Dev &d, const TrainGroup &g, const TrainBufs 
 // both networks, the gradients added to tb.grad.  A policy without train_bwd_has_out
 // gives the gradients at the last hidden layer in tb.d1, tb.d2 and keeps the output
 // layers' weight gradients to itself.
-constexpr int kTrainMaxCtas = 160, kTrainMaxSlices = 80;
+constexpr int kTrainMaxCtas = 320, kTrainMaxSlices = 80;
 bool train_bwd_has_out(const PolicyShape &p);
 size_t train_part_floats(const PolicyShape &p);
 cudaError_t launch_train_bwd(const Dev &d, const TrainGroup &g, const TrainBufs &tb, uint64_t q0,

@@ -18,8 +18,9 @@
 // the Gaussian head's action is the unclipped sample mean + sigma z rebuilt by
 // ws_advantages (the SAMPLE field), scored under the current mean and sigma.
 //
-// FP32 SIMT throughout, in chunks of kTrainChunk rows: gather the chunk's rows from
-// the ring, forward both MLPs keeping the activations, the loss head
+// In chunks of rows, on the tensor cores in three fused launches and a head where the
+// shape allows it (ws_train_fwd.cu, ws_train_bwd.cu), else layer by layer as here:
+// gather the chunk's rows from the ring, forward both MLPs keeping the activations, the loss head
 // (softmax, advantage, dL/dlogits, dL/dV), then the backward pass per layer:
 // weight gradients as row-sliced partial products summed in a fixed order
 // (deterministic), data gradients through W^T and tanh' = 1 - tanh^2.
@@ -43,22 +44,15 @@ __device__ __forceinline__ size_t ring_pos(const Dev &d, uint32_t n, size_t q0, 
   return slot0 + q % ns;
 }
 
-// The chunk's rows from the ring: obs, return, action (categorical), and for
-// PPO the held advantage and the recorded log-probability.
+// The chunk's observations from the ring (the layer-by-layer path's input).
 __global__ void k_a2c_gather(Dev d, uint32_t n, size_t q0, uint32_t rows, uint32_t slot0,
-                             uint32_t ns, int od, int ppo, TrainBufs tb) {
+                             uint32_t ns, int od, TrainBufs tb) {
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= rows) return;
   const size_t S = d.n_slots;
   size_t rowR;
   const size_t s = ring_pos(d, n, q0, i, slot0, ns, &rowR);
   for (int j = 0; j < od; ++j) tb.x[(size_t)i * od + j] = d.r_obs[(rowR * od + j) * S + s];
-  tb.ret[i] = d.r_ret[rowR * S + s];
-  if (d.env != WS_ENV_LANDSCAPE) tb.act[i] = ((const int32_t *)d.r_act)[rowR * S + s];
-  if (ppo) {
-    tb.adv[i] = d.r_adv[rowR * S + s];
-    tb.lpo[i] = d.r_logp[rowR * S + s];
-  }
 }
 
 // A = G - V(s) of the chunk's rows into the ADVANTAGE field.
@@ -68,7 +62,7 @@ __global__ void k_adv_store(Dev d, uint32_t n, size_t q0, uint32_t rows, uint32_
   if (i >= rows) return;
   size_t rowR;
   const size_t s = ring_pos(d, n, q0, i, slot0, ns, &rowR);
-  d.r_adv[rowR * d.n_slots + s] = tb.ret[i] - tb.vout[i];
+  d.r_adv[rowR * d.n_slots + s] = d.r_ret[rowR * d.n_slots + s] - tb.vout[i];
 }
 
 // The Philox normals z[j..j+3] of the Gaussian head's sample of (step k,
@@ -105,10 +99,13 @@ __global__ void k_sample_store(Dev d, uint32_t n, size_t q0, uint32_t rows, uint
   }
 }
 
-// The loss sums: reduced over the warp first, one atomic per warp (every
-// thread of the warp calls it, rows past the end with zeros).
+// The loss sums: reduced over the block first, one atomic each per block (every
+// thread calls it, rows past the end with zeros; one atomic per warp made the
+// heads 15 us per 58,368 rows, most of it the queue on these four addresses).
 __device__ __forceinline__ void add_stats(const TrainBufs &tb, double a, double b, double c,
                                           double e) {
+  __shared__ double part[4][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (int)(blockDim.x >> 5);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     a += __shfl_xor_sync(0xffffffffu, a, o);
@@ -116,11 +113,17 @@ __device__ __forceinline__ void add_stats(const TrainBufs &tb, double a, double 
     c += __shfl_xor_sync(0xffffffffu, c, o);
     e += __shfl_xor_sync(0xffffffffu, e, o);
   }
-  if ((threadIdx.x & 31) == 0) {
-    atomicAdd(tb.stats + 0, a);
-    atomicAdd(tb.stats + 1, b);
-    atomicAdd(tb.stats + 2, c);
-    atomicAdd(tb.stats + 3, e);
+  if (lane == 0) {
+    part[0][w] = a;
+    part[1][w] = b;
+    part[2][w] = c;
+    part[3][w] = e;
+  }
+  __syncthreads();
+  if (threadIdx.x < 4) {
+    double t = 0.0;
+    for (int q = 0; q < nw; ++q) t += part[threadIdx.x][q];
+    atomicAdd(tb.stats + threadIdx.x, t);
   }
 }
 
@@ -132,16 +135,19 @@ __device__ __forceinline__ void add_stats(const TrainBufs &tb, double a, double 
 // normals z (redrawn here as the sampler drew them), so d log pi / d mean =
 // z / sigma and d log pi / d raw = z^2 - 1, and dH / d raw = 1, where the
 // clamp does not hold raw.
-__global__ void k_a2c_head(Dev d, uint32_t n, size_t q0, uint32_t rows, uint32_t ns, int na,
-                           double inv_r, float c_v, float c_e, TrainBufs tb) {
+__global__ void k_a2c_head(Dev d, uint32_t n, size_t q0, uint32_t rows, uint32_t slot0, uint32_t ns,
+                           int na, double inv_r, float c_v, float c_e, TrainBufs tb) {
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   double s_pg = 0.0, s_v = 0.0, s_h = 0.0;  // rows past the end add zeros
+  size_t pos = 0, rowR = 0;                  // the row's place in the ring
+  if (i < rows) pos = ring_pos(d, n, q0, i, slot0, ns, &rowR);
+  pos += rowR * d.n_slots;
   if (i < rows && d.env == WS_ENV_LANDSCAPE) {  // one group: every slot
     const int D = (int)d.dim;
     const size_t q = q0 + i;
     const uint32_t k = (uint32_t)(d.k[0] - n + q / ns), e = (uint32_t)(q % ns);
     float *o = tb.out + (size_t)i * 2 * D;
-    const float V = tb.vout[i], G = tb.ret[i], A = G - V;
+    const float V = tb.vout[i], G = d.r_ret[pos], A = G - V;
     const float half_log_2pi = 0.91893853320467274f;
     float logp = 0.f, H = 0.f;
     for (int j = 0; j < D; j += 4) {
@@ -173,8 +179,8 @@ __global__ void k_a2c_head(Dev d, uint32_t n, size_t q0, uint32_t rows, uint32_t
       const float lp = (lg[c] - m) - lS;
       H -= expf(lp) * lp;
     }
-    const float V = tb.vout[i], G = tb.ret[i], A = G - V;
-    const int a = tb.act[i];
+    const float V = tb.vout[i], G = d.r_ret[pos], A = G - V;
+    const int a = ((const int32_t *)d.r_act)[pos];
     const float lpa = (lg[a] - m) - lS;
     for (int c = 0; c < na; ++c) {
       const float lp = (lg[c] - m) - lS, p = expf(lp);
@@ -207,30 +213,31 @@ __device__ __forceinline__ void ppo_ratio(float lp, float lpo, float A, float ep
   s_c = fabsf(rho - 1.f) > eps ? 1.0 : 0.0;
 }
 
-__global__ void k_ppo_head(Dev d, uint32_t n, size_t q0, uint32_t rows, uint32_t ns, int na,
-                           double inv_r, float eps, float c_v, float c_e, TrainBufs tb) {
+__global__ void k_ppo_head(Dev d, uint32_t n, size_t q0, uint32_t rows, uint32_t slot0, uint32_t ns,
+                           int na, double inv_r, float eps, float c_v, float c_e, TrainBufs tb) {
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   double s_pg = 0.0, s_v = 0.0, s_h = 0.0, s_c = 0.0;
+  size_t slot = 0, rowR = 0;  // the row's place in the ring
+  if (i < rows) slot = ring_pos(d, n, q0, i, slot0, ns, &rowR);
+  const size_t pos = rowR * d.n_slots + slot;
   if (i < rows && d.env == WS_ENV_LANDSCAPE) {  // one group: every slot
     const int D = (int)d.dim;
-    size_t rowR;
-    const size_t s = ring_pos(d, n, q0, i, 0, ns, &rowR);
     float *o = tb.out + (size_t)i * 2 * D;
     const float half_log_2pi = 0.91893853320467274f;
     float lp = 0.f, H = 0.f;
     for (int j = 0; j < D; ++j) {
       const float ls = fminf(fmaxf(o[D + j], -5.0f), 2.0f);
-      const float y = (d.r_sample[(rowR * D + j) * d.n_slots + s] - o[j]) / expf(ls);
+      const float y = (d.r_sample[(rowR * D + j) * d.n_slots + slot] - o[j]) / expf(ls);
       lp += -0.5f * y * y - ls - half_log_2pi;
       H += ls + 0.5f + half_log_2pi;
     }
-    const float V = tb.vout[i], G = tb.ret[i], A = tb.adv[i];
+    const float V = tb.vout[i], G = d.r_ret[pos], A = d.r_adv[pos];
     float rho, g;
-    ppo_ratio(lp, tb.lpo[i], A, eps, rho, g, s_pg, s_c);
+    ppo_ratio(lp, d.r_logp[pos], A, eps, rho, g, s_pg, s_c);
     for (int j = 0; j < D; ++j) {
       const float raw = o[D + j];
       const float ls = fminf(fmaxf(raw, -5.0f), 2.0f), sig = expf(ls);
-      const float y = (d.r_sample[(rowR * D + j) * d.n_slots + s] - o[j]) / sig;
+      const float y = (d.r_sample[(rowR * D + j) * d.n_slots + slot] - o[j]) / sig;
       const bool free_ls = raw > -5.0f && raw < 2.0f;
       o[j] = (float)(-g * y / sig * inv_r);
       o[D + j] = free_ls ? (float)((-g * (y * y - 1.f) - c_e) * inv_r) : 0.f;
@@ -250,10 +257,10 @@ __global__ void k_ppo_head(Dev d, uint32_t n, size_t q0, uint32_t rows, uint32_t
       const float lp = (lg[c] - m) - lS;
       H -= expf(lp) * lp;
     }
-    const float V = tb.vout[i], G = tb.ret[i], A = tb.adv[i];
-    const int a = tb.act[i];
+    const float V = tb.vout[i], G = d.r_ret[pos], A = d.r_adv[pos];
+    const int a = ((const int32_t *)d.r_act)[pos];
     float rho, g;
-    ppo_ratio((lg[a] - m) - lS, tb.lpo[i], A, eps, rho, g, s_pg, s_c);
+    ppo_ratio((lg[a] - m) - lS, d.r_logp[pos], A, eps, rho, g, s_pg, s_c);
     for (int c = 0; c < na; ++c) {
       const float lp = (lg[c] - m) - lS, p = expf(lp);
       lg[c] = (float)((g * (p - (c == a ? 1.f : 0.f)) + c_e * p * (lp + H)) * inv_r);
@@ -903,10 +910,6 @@ size_t train_layout(uint8_t *base, const PolicyShape &pol, TrainBufs *t) {
   };
   TrainBufs b{};
   b.x = (float *)take(CH * w0 * 4);
-  b.ret = (float *)take(CH * 4);
-  b.act = (int32_t *)take(CH * 4);
-  b.adv = (float *)take(CH * 4);
-  b.lpo = (float *)take(CH * 4);
   b.h1 = (float *)take(CH * H0 * 4);    // actor activations
   b.h2 = (float *)take(CH * H1 * 4);
   b.out = (float *)take(CH * NA * 4);   // logits, then dL/dlogits
@@ -952,14 +955,15 @@ void run_update(const Dev &d, const TrainBufs &tb, const TrainGroup *groups, int
     if (use_train_tc(d, G.pol)) launch_train_pack(G, tb.image, st);
     for (size_t q0 = 0; q0 < R; q0 += CH) {
       const int rows = (int)((R - q0) < CH ? (R - q0) : CH);
-      k_a2c_gather<<<nblk(rows, 256), 256, 0, st>>>(d, n, q0, (uint32_t)rows, G.slot0, G.n_slots,
-                                                    G.pol.w[0], ppo ? 1 : 0, tb);
+      if (!use_train_tc(d, G.pol))
+        k_a2c_gather<<<nblk(rows, 256), 256, 0, st>>>(d, n, q0, (uint32_t)rows, G.slot0, G.n_slots,
+                                                      G.pol.w[0], tb);
       chunk_forward(d, tb, G, n, q0, rows, false, st);
       if (ppo)
-        k_ppo_head<<<nblk(rows, 256), 256, 0, st>>>(d, n, q0, (uint32_t)rows, G.n_slots,
+        k_ppo_head<<<nblk(rows, 256), 256, 0, st>>>(d, n, q0, (uint32_t)rows, G.slot0, G.n_slots,
                                                     G.pol.w[3], inv_r, eps, c_v, c_e, tb);
       else
-        k_a2c_head<<<nblk(rows, 256), 256, 0, st>>>(d, n, q0, (uint32_t)rows, G.n_slots,
+        k_a2c_head<<<nblk(rows, 256), 256, 0, st>>>(d, n, q0, (uint32_t)rows, G.slot0, G.n_slots,
                                                     G.pol.w[3], inv_r, c_v, c_e, tb);
       chunk_backward(d, tb, G, n, q0, rows, st);
     }
@@ -991,8 +995,9 @@ void launch_advantages(const Dev &d, const TrainBufs &tb, const TrainGroup *grou
     if (use_train_tc(d, G.pol)) launch_train_pack(G, tb.image, st);
     for (size_t q0 = 0; q0 < R; q0 += CH) {
       const int rows = (int)((R - q0) < CH ? (R - q0) : CH);
-      k_a2c_gather<<<nblk(rows, 256), 256, 0, st>>>(d, n, q0, (uint32_t)rows, G.slot0, G.n_slots,
-                                                    G.pol.w[0], 0, tb);
+      if (!use_train_tc(d, G.pol))
+        k_a2c_gather<<<nblk(rows, 256), 256, 0, st>>>(d, n, q0, (uint32_t)rows, G.slot0, G.n_slots,
+                                                      G.pol.w[0], tb);
       chunk_forward(d, tb, G, n, q0, rows, !both, st);
       k_adv_store<<<nblk(rows, 256), 256, 0, st>>>(d, n, q0, (uint32_t)rows, G.slot0, G.n_slots,
                                                    tb);

@@ -38,42 +38,49 @@ struct BNets {
 template <int H, int XP, int OUT>
 struct BwdSmem {
   using G = Geo<H>;
-  static constexpr int NO = OUT > 1 ? OUT : 1;         // the wider of the two networks
-  static constexpr int NG3 = kCT / H;                  // row groups of dW3
-  static constexpr int SL1 = kCT * (XP + 1) * 4;       // dW1's group sums, over the operand tiles
+  static constexpr int SL1 = kCT * (XP + 1) * 4;       // dW1's group sums, over the operand tile
   static constexpr int REG = G::REG > SL1 ? G::REG : SL1;
   static constexpr int OFF_B = (REG + 1023) / 1024 * 1024;
   static constexpr int OFF_BAR = OFF_B + G::B_BYTES;
   static constexpr int OFF_X = OFF_BAR + ((int)sizeof(Bars) + 15) / 16 * 16;  // [128][XP]
-  static constexpr int OFF_D = OFF_X + kRows * XP * 4;                          // [128][NO]
-  static constexpr int OFF_W3 = OFF_D + (kRows * NO * 4 + 15) / 16 * 16;        // [NO][H]
-  static constexpr int OFF_S3 = OFF_W3 + NO * H * 4;                            // [NG3][H][NO]
-  static constexpr int OFF_A3 = OFF_S3 + NG3 * H * NO * 4;                      // [(H + 1) NO]
-  static constexpr int OFF_A1 = OFF_A3 + ((H + 1) * NO * 4 + 15) / 16 * 16;     // [(XP + 1) H]
+  static constexpr int OFF_D = OFF_X + kRows * XP * 4;                          // [128][OUT]
+  static constexpr int OFF_W3 = OFF_D + (kRows * OUT * 4 + 15) / 16 * 16;       // [OUT][H]
+  static constexpr int OFF_A3 = OFF_W3 + OUT * H * 4;                           // [(H + 1) OUT]
+  static constexpr int OFF_A1 = OFF_A3 + ((H + 1) * OUT * 4 + 15) / 16 * 16;    // [(XP + 1) H]
   static constexpr int WITH_A1 = OFF_A1 + (XP + 1) * H * 4 + 1024;
-  static constexpr bool A1_SMEM = WITH_A1 <= 232448;  // else the dW1 sums stay in global memory
+  static constexpr bool A1_SMEM = WITH_A1 <= kSmemPerCta;  // else the dW1 sums stay in global memory
   static constexpr int BYTES = A1_SMEM ? WITH_A1 : OFF_A1 + 1024;
-  static_assert(BYTES <= 232448, "shared memory over the 227 KB per-CTA limit");
+  static_assert(BYTES <= kSmemPerCta, "shared memory of half an SM");
 };
 
 // One tile of one network by the compute warps; a1, a3 the CTA's running sums.
-template <int H, int XP, int OUT, int NO>
+template <int H, int XP, int OUT, bool A1S>
 __device__ __forceinline__ bool bwd_tile(const BNet &net, Bars *bars, uint8_t *reg, const float *xs,
-                                         float *ds, const float *w3t, float *s3, float *a1, float *a3,
-                                         int in, int rows, int tile, uint32_t tmem, uint32_t ph_acc) {
+                                         float *ds, const float *w3t, float *a1, float *a3, int in,
+                                         int rows, int tile, uint32_t tmem, uint32_t ph_acc,
+                                         uint32_t &ph_af) {
   using G = Geo<H>;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int l16 = lane & 15, rh = lane >> 4;
   const uint32_t a = tc::smem_u32(reg);
   const size_t row0 = (size_t)tile * kRows;
   // ---- d2, one 64-unit K block at a time
+  bool okw = true;
+  const float *src = (OUT > 0 ? net.h2 : net.d2) + (row0 + warp * kWR16 + rh) * H + l16 * 4;
+  float4 hn[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) hn[i] = __ldg((const float4 *)(src + 2 * i * H));
 #pragma unroll 1
-  for (int kb = 0; kb < G::KB; ++kb) {
-    const int col = kb * 64 + l16 * 4;
+  for (int it = 0; it < 2 * G::KB; ++it) {  // half a block (eight rows per warp) at a time
+    const int kb = it >> 1, i0 = (it & 1) * 8, col = kb * 64 + l16 * 4;
     float4 h[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-      h[i] = __ldg((const float4 *)((OUT > 0 ? net.h2 : net.d2) + (row0 + warp * 8 + 2 * i + rh) * H + col));
+    for (int i = 0; i < 4; ++i) h[i] = hn[i];
+    if (it + 1 < 2 * G::KB) {  // the next half's loads run under this half's work
+      const float *nx = src + ((it + 1) & 1) * 8 * H + ((it + 1) >> 1) * 64;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) hn[i] = __ldg((const float4 *)(nx + 2 * i * H));
+    }
     float s[4][4];
 #pragma unroll
     for (int i = 0; i < 4; ++i)
@@ -85,7 +92,7 @@ __device__ __forceinline__ bool bwd_tile(const BNet &net, Bars *bars, uint8_t *r
         const float4 w = *(const float4 *)(w3t + o * H + col);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          const float dv = ds[(warp * 8 + 2 * i + rh) * OUT + o];
+          const float dv = ds[(warp * kWR16 + i0 + 2 * i + rh) * OUT + o];
           s[i][0] = fmaf(dv, w.x, s[i][0]);
           s[i][1] = fmaf(dv, w.y, s[i][1]);
           s[i][2] = fmaf(dv, w.z, s[i][2]);
@@ -93,9 +100,10 @@ __device__ __forceinline__ bool bwd_tile(const BNet &net, Bars *bars, uint8_t *r
         }
       }
     }
+    if (i0 == 0) okw = wait_block(bars, kb, ph_af) && okw;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      const int r = warp * 8 + 2 * i + rh;
+      const int r = warp * kWR16 + i0 + 2 * i + rh;
       if (OUT > 0) {
         s[i][0] *= 1.f - h[i].x * h[i].x;
         s[i][1] *= 1.f - h[i].y * h[i].y;
@@ -109,72 +117,71 @@ __device__ __forceinline__ bool bwd_tile(const BNet &net, Bars *bars, uint8_t *r
         s[i][2] = ok ? h[i].z : 0.f;
         s[i][3] = ok ? h[i].w : 0.f;
       }
-      store_a<H>(a, kb, r, l16 * 4, s[i]);
+      store_a(a, r, l16 * 4, s[i]);
     }
-    tc::fence_async_smem();
-    tc::fence_before_sync();
-    __syncwarp();
-    if (lane == 0) arrive(bars->a + kb);
+    if (i0) {
+      tc::fence_async_smem();
+      tc::fence_before_sync();
+      __syncwarp();
+      if (lane == 0) arrive(&bars->a);
+    }
   }
-  // ---- dW3 and db3 of the tile while the products run: thread (column, row group)
+  // ---- dW3 and db3 of the tile while the products run: a thread per column and share
+  // of the outputs
   if (OUT > 0) {
-    constexpr int NG = kCT / H, L = kRows / NG, O = OUT > 0 ? OUT : 1;
-    const int c = tid % H, g = tid / H;
-    float acc[O];
+    constexpr int TPC = kCT / H > 0 ? kCT / H : 1, O = (OUT + TPC - 1) / TPC > 0 ? (OUT + TPC - 1) / TPC : 1;
+    const int c = tid % H, o0 = tid / H * O;
+    if (o0 < OUT) {
+      float acc[O];
 #pragma unroll
-    for (int o = 0; o < O; ++o) acc[o] = 0.f;
-    const float *hp = net.h2 + (row0 + g * L) * H + c;
+      for (int o = 0; o < O; ++o) acc[o] = 0.f;
+      const float *hp = net.h2 + row0 * H + c;
+      constexpr int U = 16;  // loads in flight
 #pragma unroll 1
-    for (int r = 0; r < L; r += 8) {
-      float hv[8];
+      for (int r = 0; r < kRows; r += U) {
+        float hv[U];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) hv[u] = __ldg(hp + (size_t)(r + u) * H);
+        for (int u = 0; u < U; ++u) hv[u] = __ldg(hp + (size_t)(r + u) * H);
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const float *dp = ds + (g * L + r + u) * O;
+        for (int u = 0; u < U; ++u) {
+          const float *dp = ds + (r + u) * OUT + o0;
 #pragma unroll
-        for (int o = 0; o < O; ++o) acc[o] = fmaf(hv[u], dp[o], acc[o]);
+          for (int o = 0; o < O; ++o)
+            if (OUT % O == 0 || o0 + o < OUT) acc[o] = fmaf(hv[u], dp[o], acc[o]);
+        }
       }
+#pragma unroll
+      for (int o = 0; o < O; ++o)
+        if (OUT % O == 0 || o0 + o < OUT) a3[c * OUT + o0 + o] += acc[o];
     }
+    for (int o = warp; o < OUT; o += kCW) {  // db3: a warp per output
+      float t = 0.f;
 #pragma unroll
-    for (int o = 0; o < O; ++o) s3[(g * H + c) * O + o] = acc[o];
-    csync();
-    for (int v = tid; v < H * O; v += kCT) {
-      float t = s3[v];
+      for (int r = 0; r < kRows; r += 32) t += ds[(r + lane) * OUT + o];
 #pragma unroll
-      for (int q = 1; q < NG; ++q) t += s3[q * (H * O) + v];
-      a3[v] += t;
-    }
-    if (warp < O || O > kCW) {
-      for (int o = warp; o < O; o += kCW) {  // db3: a warp per output
-        float t = 0.f;
-#pragma unroll
-        for (int r = 0; r < kRows; r += 32) t += ds[(r + lane) * O + o];
-#pragma unroll
-        for (int m = 16; m > 0; m >>= 1) t += __shfl_xor_sync(0xffffffffu, t, m);
-        if (lane == 0) a3[H * O + o] += t;
-      }
+      for (int m = 16; m > 0; m >>= 1) t += __shfl_xor_sync(0xffffffffu, t, m);
+      if (lane == 0) a3[H * OUT + o] += t;
     }
   }
   // ---- d1 and dW1
-  const bool ok = call(tc::mbar_wait(&bars->acc, ph_acc, tc::kDrainNs));
+  const bool ok = call(tc::mbar_wait(&bars->acc, ph_acc, tc::kDrainNs) && okw);
   if (!ok) return false;
   tc::fence_after_sync();
   float *ct = (float *)reg;
 #pragma unroll 1
   for (int c0 = 0; c0 < H; c0 += G::CTW) {
-    constexpr int LPR = G::CTW / 4, RPW = 32 / LPR, NI = 8 / RPW;  // lanes per row, rows per access
+    constexpr int LPR = G::CTW / 4, RPW = 32 / LPR, NI = kWR16 / RPW;  // lanes per row, rows per access
     const int c = (lane % LPR) * 4;
     float4 h[NI];  // the activations' loads in flight while the accumulator is staged
 #pragma unroll
     for (int i = 0; i < NI; ++i)
-      h[i] = __ldg((const float4 *)(net.h1 + (row0 + warp * 8 + i * RPW + lane / LPR) * H + c0 + c));
+      h[i] = __ldg((const float4 *)(net.h1 + (row0 + warp * kWR16 + i * RPW + lane / LPR) * H + c0 + c));
     stage_acc<H>(tmem, ct, c0, warp, lane);
     tc::fence_before_sync();
     csync();
 #pragma unroll
     for (int i = 0; i < NI; ++i) {
-      float4 *p = (float4 *)(ct + (warp * 8 + i * RPW + lane / LPR) * G::CP + c);
+      float4 *p = (float4 *)(ct + (warp * kWR16 + i * RPW + lane / LPR) * G::CP + c);
       float4 v = *p;
       v.x *= 1.f - h[i].x * h[i].x;
       v.y *= 1.f - h[i].y * h[i].y;
@@ -212,7 +219,10 @@ __device__ __forceinline__ bool bwd_tile(const BNet &net, Bars *bars, uint8_t *r
       float t = 0.f;
 #pragma unroll
       for (int u = 0; u < NG; ++u) t += sl[(u * (XP + 1) + kk) * G::CTW + q];
-      a1[k * H + c0 + q] += t;
+      if (A1S)
+        a1[k * H + c0 + q] += t;
+      else
+        atomicAdd(a1 + k * H + c0 + q, t);  // (this thread's alone: no wait for the old value)
     }
     csync();
   }
@@ -220,7 +230,7 @@ __device__ __forceinline__ bool bwd_tile(const BNet &net, Bars *bars, uint8_t *r
 }
 
 template <int H, int XP, int OUT>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kThreads, 2)
     k_train_bwd(Dev d, Rows rw, int in, const __grid_constant__ BNets nets) {
   using G = Geo<H>;
   using S = BwdSmem<H, XP, OUT>;
@@ -229,7 +239,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint8_t *sm = smem_raw + ((1024u - (raw & 1023u)) & 1023u);
   Bars *bars = (Bars *)(sm + S::OFF_BAR);
   float *xs = (float *)(sm + S::OFF_X), *ds = (float *)(sm + S::OFF_D);
-  float *w3t = (float *)(sm + S::OFF_W3), *s3 = (float *)(sm + S::OFF_S3), *a3 = (float *)(sm + S::OFF_A3);
+  float *w3t = (float *)(sm + S::OFF_W3), *a3 = (float *)(sm + S::OFF_A3);
   const int tid = threadIdx.x, warp = tid >> 5;
   if (tid == 0) bars_init(bars);
   if (warp == kCW) tc::tmem_alloc(&bars->tmem, H);
@@ -254,7 +264,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     __syncwarp();
   } else {
-    uint32_t ph = 0;
+    uint32_t ph = 0, ph_af = 0;
+    constexpr int XV = (XP + kXT - 1) / kXT;
     for (int q = 0; q < nets.count && ok; ++q) {
       const BNet &net = nets.n[q];
       const int no = q == 0 ? OUT : (OUT > 0 ? 1 : 0);  // 0: no output layer here
@@ -264,21 +275,24 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int i = tid; i < (in + 1) * H; i += kCT) a1[i] = 0.f;
       for (int i = tid; i < (H + 1) * no; i += kCT) a3[i] = 0.f;
       for (int i = tid; i < no * H; i += kCT) w3t[i] = __ldg(net.W3 + (i % H) * no + i / H);
-      const int mine = my_tiles(tiles, q);
+      const int mine = my_tiles(tiles, q), t0 = first_tile(tiles, q);
+      float xn[XV];
+      if (mine > 0) load_x(d, rw, t0, in, xn);
       for (int t = 0; t < mine && ok; ++t) {
-        const int tile = first_tile(tiles, q) + t * (int)gridDim.x;
-        gather_x(d, rw, tile, in, XP, xs);
+        const int tile = t0 + t * (int)gridDim.x;
+        store_x(xn, XP, xs);
         for (int i = tid; i < kRows * no; i += kCT) {
           const int r = tile * kRows + i / (no > 0 ? no : 1);
           ds[i] = r < (int)rw.rows ? net.dout[(size_t)tile * kRows * no + i] : 0.f;
         }
         csync();
+        if (t + 1 < mine) load_x(d, rw, tile + (int)gridDim.x, in, xn);
         if (q == 0)
-          ok = bwd_tile<H, XP, OUT, S::NO>(net, bars, sm, xs, ds, w3t, s3, a1, a3, in, (int)rw.rows,
-                                           tile, tmem, ph);
+          ok = bwd_tile<H, XP, OUT, S::A1_SMEM>(net, bars, sm, xs, ds, w3t, a1, a3, in, (int)rw.rows,
+                                                tile, tmem, ph, ph_af);
         else
-          ok = bwd_tile<H, XP, (OUT > 0 ? 1 : 0), S::NO>(net, bars, sm, xs, ds, w3t, s3, a1, a3, in,
-                                                         (int)rw.rows, tile, tmem, ph);
+          ok = bwd_tile<H, XP, (OUT > 0 ? 1 : 0), S::A1_SMEM>(net, bars, sm, xs, ds, w3t, a1, a3, in,
+                                                              (int)rw.rows, tile, tmem, ph, ph_af);
         ph ^= 1u;
       }
       csync();
@@ -302,6 +316,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 // warps (two rows each) load float4s of both arrays one stage ahead and store them
 // as hi and lo tiles in the 128B-swizzled MN-major layout: 64 units of a row are one
 // 128-byte line, eight rows a swizzle atom, four atoms (32 rows) a 64-unit block.
+constexpr int kWW = 16, kWC = 32 * kWW, kWT = kWC + 32;  // loader warps, their threads, and the MMA warp
 constexpr int kWR = 32;   // rows per stage
 constexpr int kWS = 4;    // stages
 template <int H>
@@ -315,7 +330,7 @@ struct WGeo {
   static constexpr int CT = kRows * 132 * 4;            // output staging over the stages
   static constexpr int REG = kWS * STAGE > CT ? kWS * STAGE : CT;
   static constexpr int OFF_CS = REG;                    // [16][H] column sums
-  static constexpr int OFF_BAR = OFF_CS + kCW * H * 4;
+  static constexpr int OFF_BAR = OFF_CS + kWW * H * 4;
   static constexpr int SMEM = OFF_BAR + 128 + 1024;
   static_assert(SMEM <= 232448, "shared memory over the 227 KB per-CTA limit");
 };
@@ -341,8 +356,23 @@ __device__ __forceinline__ void store_mn(uint32_t base, int r, int c, const floa
   sts64(o + lo_off, lo[0], lo[1]);
 }
 
+// Barrier (and AND vote) of the loader warps.
+__device__ __forceinline__ void wsync() { asm volatile("bar.sync 1, 512;" ::: "memory"); }
+__device__ __forceinline__ bool wall(bool v) {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.u32 p, %1, 0;\n\t"
+      "bar.red.and.pred q, 1, 512, p;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(r)
+      : "r"((uint32_t)v)
+      : "memory");
+  return r != 0;
+}
+
 template <int H>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kWT, 1)
     k_train_wgrad(const __grid_constant__ WNet n0, const __grid_constant__ WNet n1, int rows, int per,
                   uint32_t *err) {
   using G = WGeo<H>;
@@ -359,22 +389,22 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int ns = re > rb ? (re - rb + kWR - 1) / kWR : 0;
   if (tid == 0) {
     for (int i = 0; i < kWS; ++i) {
-      tc::mbar_init(full + i, kCW);
+      tc::mbar_init(full + i, kWW);
       tc::mbar_init(empty + i, 1);
     }
     tc::mbar_init(done, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (H < 128)  // the operand's unused half
-    for (int i = tid; i < kWS * G::STAGE / 16; i += kThreads) ((uint4 *)sm)[i] = make_uint4(0, 0, 0, 0);
-  if (warp == kCW) tc::tmem_alloc(holder, H);
+    for (int i = tid; i < kWS * G::STAGE / 16; i += kWT) ((uint4 *)sm)[i] = make_uint4(0, 0, 0, 0);
+  if (warp == kWW) tc::tmem_alloc(holder, H);
   tc::fence_async_smem();
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = *holder;
   bool ok = true;
-  if (warp == kCW) {
+  if (warp == kWW) {
     if (lane == 0 && ns > 0) {
       for (int s = 0; s < ns && ok; ++s) {
         const int b = s % kWS;
@@ -407,14 +437,14 @@ __global__ void __launch_bounds__(kThreads, 1)
     // warp w: rows 2 w, 2 w + 1 of a stage; a lane's columns: 128 j + 4 lane (H >=
     // 128), or 4 (lane % 16) of row 2 w + lane / 16 (H = 64)
     constexpr int NB = H >= 128 ? 2 * (H / 128) : 1, NA = H >= 128 ? 2 : 1;
-    float4 va[NA], vb[NB];
+    float4 va[2][NA], vb[2][NB];  // the next two stages, in flight
     float cs[H >= 128 ? H / 128 : 1][4];
 #pragma unroll
     for (int j = 0; j < (H >= 128 ? H / 128 : 1); ++j)
 #pragma unroll
       for (int q = 0; q < 4; ++q) cs[j][q] = 0.f;
     const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-    auto load = [&](int s) {
+    auto load = [&](int s, float4 (&va)[NA], float4 (&vb)[NB]) {
       const int r0 = rb + s * kWR + warp * 2;
       if (H >= 128) {
 #pragma unroll
@@ -432,13 +462,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         vb[0] = r < re ? __ldg((const float4 *)(net.d2 + (size_t)r * H + 4 * (lane & 15))) : zero;
       }
     };
-    if (ns > 0) load(0);
-    for (int s = 0; s < ns && ok; ++s) {
-      const int b = s % kWS;
-      if (s >= kWS) ok = tc::mbar_wait(empty + b, (uint32_t)(s / kWS - 1) & 1u, tc::kDrainNs);
-      ok = __all_sync(0xffffffffu, ok);
-      if (!ok) break;
-      const uint32_t st = sb + (uint32_t)(b * G::STAGE);
+    auto put = [&](int s, const float4 (&va)[NA], const float4 (&vb)[NB]) {
+      const uint32_t st = sb + (uint32_t)((s % kWS) * G::STAGE);
       if (H >= 128) {
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
@@ -463,10 +488,24 @@ __global__ void __launch_bounds__(kThreads, 1)
         cs[0][2] += vb[0].z;
         cs[0][3] += vb[0].w;
       }
-      if (s + 1 < ns) load(s + 1);
-      tc::fence_async_smem();
-      __syncwarp();
-      if (lane == 0) arrive(full + b);
+    };
+    if (ns > 0) load(0, va[0], vb[0]);
+    if (ns > 1) load(1, va[1], vb[1]);
+    for (int s0 = 0; s0 < ns && ok; s0 += 2) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {  // the register buffers by compile-time index
+        const int s = s0 + h;
+        if (s >= ns || !ok) break;
+        const int b = s % kWS;
+        if (s >= kWS) ok = tc::mbar_wait(empty + b, (uint32_t)(s / kWS - 1) & 1u, tc::kDrainNs);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        put(s, va[h], vb[h]);
+        if (s + 2 < ns) load(s + 2, va[h], vb[h]);
+        tc::fence_async_smem();
+        __syncwarp();
+        if (lane == 0) arrive(full + b);
+      }
     }
     float *csum = (float *)(sm + G::OFF_CS);
     if (H >= 128) {
@@ -482,14 +521,14 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     float *out = net.part + (size_t)slice * ((size_t)(H + 1) * H);
     if (ns > 0) ok = tc::mbar_wait(done, 0, tc::kDrainNs) && ok;
-    ok = call(ok);
+    ok = wall(ok);
     if (ok) {
       tc::fence_after_sync();
       if (m0 == 0)
-        for (int c = tid; c < H; c += kCT) {
+        for (int c = tid; c < H; c += kWC) {
           float t = csum[c];
 #pragma unroll
-          for (int w = 1; w < kCW; ++w) t += csum[w * H + c];
+          for (int w = 1; w < kWW; ++w) t += csum[w * H + c];
           out[(size_t)H * H + c] = t;
         }
       float *ct = (float *)sm;
@@ -512,26 +551,29 @@ __global__ void __launch_bounds__(kThreads, 1)
             *(float4 *)(o + i) = make_float4(__uint_as_float(z[i]), __uint_as_float(z[i + 1]),
                                              __uint_as_float(z[i + 2]), __uint_as_float(z[i + 3]));
         }
-        csync();
-        for (int i = tid; i < G::MC * CW / 4; i += kCT) {
+        wsync();
+        for (int i = tid; i < G::MC * CW / 4; i += kWC) {
           const int m = i / (CW / 4), c = (i % (CW / 4)) * 4;
           *(float4 *)(out + (size_t)(m0 + m) * H + c0 + c) = *(const float4 *)(ct + m * 132 + c);
         }
-        csync();
+        wsync();
       }
     }
   }
   tc::fence_before_sync();
   __syncthreads();
-  if (warp == kCW) {
+  if (warp == kWW) {
     tc::fence_after_sync();
     tc::tmem_dealloc(tmem, H);
   }
 }
 
 // ------------------------------------------------------------ slice sums
-// grad[i] += sum_z P[z stride + i], z in a fixed order (as k_reduce_slices), for all
-// layers of both networks in one launch.
+// grad[i] += sum_z P[z len + i], z in a fixed order, for all layers of both networks
+// in one launch: a block per 32 consecutive i (eight lanes of four where every slice
+// starts on 16 bytes), 64 groups of lanes over the slices z, z + 64, ..., then the
+// groups' sums in order, eight and eight.  Short chains and many blocks: the kernel
+// is a latency of two loads and three barriers over the read of the partial sums.
 struct Seg {
   const float *P;
   float *grad;
@@ -542,25 +584,48 @@ struct Segs {
   Seg s[6];
   int count;
 };
-__global__ __launch_bounds__(256) void k_train_reduce(const __grid_constant__ Segs segs) {
-  __shared__ float part[8][32];
+__global__ __launch_bounds__(512) void k_train_reduce(const __grid_constant__ Segs segs) {
+  __shared__ float4 part[64][8];
+  __shared__ float part2[8][32];
   int q = 0;
   while (q + 1 < segs.count && blockIdx.x >= segs.s[q + 1].block0) ++q;
-  const Seg sg = segs.s[q];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const size_t i = (size_t)(blockIdx.x - sg.block0) * 32 + lane;
-  float s = 0.f;
-  if (i < sg.len) {
-#pragma unroll 10
-    for (int z = w; z < sg.nz; z += 8) s += __ldcs(sg.P + (size_t)z * sg.len + i);
+  const Seg &sg = segs.s[q];
+  const int l = threadIdx.x & 7, g = threadIdx.x >> 3;
+  const uint32_t i0 = (blockIdx.x - sg.block0) * 32, i = i0 + 4 * l;
+  const bool vec = (sg.len & 3) == 0 && ((uintptr_t)sg.P & 15) == 0;
+  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 3
+  for (int z = g; z < sg.nz; z += 64) {
+    const float *p = sg.P + (size_t)z * sg.len + i;
+    if (vec && i < sg.len) {
+      const float4 v = __ldcs((const float4 *)p);
+      s.x += v.x;
+      s.y += v.y;
+      s.z += v.z;
+      s.w += v.w;
+    } else if (!vec) {
+      if (i < sg.len) s.x += __ldcs(p);
+      if (i + 1 < sg.len) s.y += __ldcs(p + 1);
+      if (i + 2 < sg.len) s.z += __ldcs(p + 2);
+      if (i + 3 < sg.len) s.w += __ldcs(p + 3);
+    }
   }
-  part[w][lane] = s;
+  part[g][l] = s;
   __syncthreads();
-  if (w == 0 && i < sg.len) {
-    float t = sg.grad[i];
+  const float *pf = (const float *)part;
+  const int c = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if (w < 8) {
+    float t = pf[8 * w * 32 + c];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) t += part[k][lane];
-    sg.grad[i] = t;
+    for (int k = 1; k < 8; ++k) t += pf[(8 * w + k) * 32 + c];
+    part2[w][c] = t;
+  }
+  __syncthreads();
+  if (w == 0 && i0 + c < sg.len) {
+    float t = sg.grad[i0 + c];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) t += part2[k][c];
+    sg.grad[i0 + c] = t;
   }
 }
 
@@ -568,7 +633,7 @@ int sm_count() {
   int dev = 0, sms = 148;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  return sms < kTrainMaxCtas ? sms : kTrainMaxCtas;
+  return sms < kTrainMaxCtas / 2 ? sms : kTrainMaxCtas / 2;
 }
 
 template <int H, int XP, int OUT>
@@ -603,7 +668,7 @@ cudaError_t run_wgrad(const WNet &a, const WNet &c, int rows, int slices, int pe
   using G = WGeo<H>;
   cudaError_t e = cudaFuncSetAttribute(k_train_wgrad<H>, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM);
   if (e != cudaSuccess) return e;
-  k_train_wgrad<H><<<dim3((unsigned)slices, G::MH, 2), kThreads, G::SMEM, st>>>(a, c, rows, per, err);
+  k_train_wgrad<H><<<dim3((unsigned)slices, G::MH, 2), kWT, G::SMEM, st>>>(a, c, rows, per, err);
   return cudaGetLastError();
 }
 
@@ -628,7 +693,7 @@ cudaError_t launch_train_bwd(const Dev &d, const TrainGroup &g, const TrainBufs 
   const int H = p.w[1], in = p.w[0], out = p.w[3];
   const bool has = train_bwd_has_out(p);
   const int sms = sm_count(), tiles = (int)((rows + kRows - 1) / kRows);
-  const int grid = 2 * tiles < sms ? 2 * tiles : sms;
+  const int grid = tiles < sms ? 2 * tiles : 2 * sms;
   const size_t ib = (size_t)4 * H * H;
   // partials: per network p1, p3 [grid], then the dW2 slices
   const size_t l1 = (size_t)(in + 1) * H, l2 = (size_t)(H + 1) * H, l3a = (size_t)(H + 1) * out, l3c = H + 1;
@@ -677,7 +742,7 @@ cudaError_t launch_train_bwd(const Dev &d, const TrainGroup &g, const TrainBufs 
     seg(p3a, ga + g.pol.layer_offset(2), grid, l3a);
     seg(p3c, gc + g.crit.layer_offset(2), grid, l3c);
   }
-  k_train_reduce<<<blocks, 256, 0, st>>>(s);
+  k_train_reduce<<<blocks, 512, 0, st>>>(s);
   return cudaGetLastError();
 }
 

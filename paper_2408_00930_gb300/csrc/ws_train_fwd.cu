@@ -35,8 +35,16 @@ struct FwdSmem {
   using G = Geo<H>;
   static constexpr int OFF_B = (G::REG + 1023) / 1024 * 1024;
   static constexpr int OFF_BAR = OFF_B + G::B_BYTES;
-  static constexpr int OFF_X = OFF_BAR + (int)sizeof(Bars) + 16;
-  static int bytes(int xp) { return OFF_X + kRows * xp * 4 + 1024; }
+  static constexpr int OFF_X = OFF_BAR + ((int)sizeof(Bars) + 15) / 16 * 16;
+  // after the observations: W1, b1, b2 and W3 of the network in work, where they fit
+  static int off_w(int xp) { return OFF_X + kRows * xp * 4; }
+  static int w_floats(int in, int out) { return (in + 2 + out) * H; }
+  static bool w_fits(int in, int xp, int out) {
+    return off_w(xp) + w_floats(in, out) * 4 + 1024 <= kSmemPerCta;
+  }
+  static int bytes(int in, int xp, int out) {
+    return off_w(xp) + (w_fits(in, xp, out) ? w_floats(in, out) * 4 : 0) + 1024;
+  }
 };
 
 // W2[k][n] (FP32, row-major) as the MMA's B operand, hi and lo per K = 16 chunk:
@@ -60,23 +68,23 @@ __global__ void k_pack_w2(const float *__restrict__ W2a, const float *__restrict
   }
 }
 
-// Output layer over one staged pass: thread (row, g) sums units g CTW / 4 .. of the
+// Output layer over one staged pass: thread (row, g) sums units g CTW / 2 .. of the
 // pass into acc (FP32 FMAs in unit order).
 template <int H, int OUT>
 __device__ __forceinline__ void out_pass(const float *ct, const float *__restrict__ W3, int c0,
                                          float (&acc)[OUT]) {
   using G = Geo<H>;
   const int r = threadIdx.x & 127, g = threadIdx.x >> 7;
-  constexpr int L = G::CTW / 4;
+  constexpr int L = G::CTW / (kCT / kRows);
   const float *h = ct + r * G::CP + g * L;
   const float4 *w = (const float4 *)(W3 + (size_t)(c0 + g * L) * OUT);  // 16-byte aligned: c0 + g L is a multiple of 16
-#pragma unroll 2
+#pragma unroll(OUT <= 3 ? 4 : 1)
   for (int k = 0; k < L; k += 4) {
     const float4 hv = *(const float4 *)(h + k);
     float wv[4 * OUT];
 #pragma unroll
     for (int q = 0; q < OUT; ++q) {
-      const float4 v = __ldg(w + (k / 4) * OUT + q);
+      const float4 v = w[(k / 4) * OUT + q];
       wv[4 * q] = v.x;
       wv[4 * q + 1] = v.y;
       wv[4 * q + 2] = v.z;
@@ -94,53 +102,65 @@ __device__ __forceinline__ void out_pass(const float *ct, const float *__restric
 
 // One tile of one network by the compute warps (OUT = 0: no output layer here).
 // Returns false if the accumulator's wait ran out.
-template <int H, int OUT>
-__device__ __forceinline__ bool fwd_tile(const Net &net, Bars *bars, uint8_t *reg, const float *xs,
-                                         int in, int xp, int tile, uint32_t tmem, uint32_t ph_acc) {
+template <int H, int OUT, int XV>
+__device__ __forceinline__ bool fwd_tile(const Net &net, Bars *bars, uint8_t *reg, float *xs, int in,
+                                         int xp, int tile, uint32_t tmem, uint32_t ph_acc,
+                                         uint32_t &ph_af, const Dev &d, const Rows &rw, int next) {
   using G = Geo<H>;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int l16 = lane & 15, rh = lane >> 4;
   const uint32_t a = tc::smem_u32(reg);
   const size_t row0 = (size_t)tile * kRows;
   // ---- layer 1, one 64-unit K block at a time
+  bool okw = true;
 #pragma unroll 1
   for (int kb = 0; kb < G::KB; ++kb) {
     const int col = kb * 64 + l16 * 4;
-    float z[4][4];
+    const float4 b = *(const float4 *)(net.b1 + col);
+#pragma unroll 1
+    for (int i0 = 0; i0 < kWR16; i0 += 8) {  // eight rows at a time
+      float z[4][4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < 4; ++i)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) z[i][j] = 0.f;
+        for (int j = 0; j < 4; ++j) z[i][j] = 0.f;
+      const float *xr = xs + (warp * kWR16 + i0 + rh) * xp;
 #pragma unroll 4
-    for (int k = 0; k < in; ++k) {
-      const float4 w = __ldg((const float4 *)(net.W1 + (size_t)k * H + col));
+      for (int k = 0; k < in; ++k) {
+        const float4 w = *(const float4 *)(net.W1 + k * H + col);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float x = xr[2 * i * xp + k];
+          z[i][0] = fmaf(x, w.x, z[i][0]);
+          z[i][1] = fmaf(x, w.y, z[i][1]);
+          z[i][2] = fmaf(x, w.z, z[i][2]);
+          z[i][3] = fmaf(x, w.w, z[i][3]);
+        }
+      }
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const float x = xs[(warp * 8 + 2 * i + rh) * xp + k];
-        z[i][0] = fmaf(x, w.x, z[i][0]);
-        z[i][1] = fmaf(x, w.y, z[i][1]);
-        z[i][2] = fmaf(x, w.z, z[i][2]);
-        z[i][3] = fmaf(x, w.w, z[i][3]);
+        z[i][0] = tanhf(z[i][0] + b.x);
+        z[i][1] = tanhf(z[i][1] + b.y);
+        z[i][2] = tanhf(z[i][2] + b.z);
+        z[i][3] = tanhf(z[i][3] + b.w);
       }
-    }
-    const float4 b = __ldg((const float4 *)(net.b1 + col));
+      if (i0 == 0) okw = wait_block(bars, kb, ph_af) && okw;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int r = warp * 8 + 2 * i + rh;
-      z[i][0] = tanhf(z[i][0] + b.x);
-      z[i][1] = tanhf(z[i][1] + b.y);
-      z[i][2] = tanhf(z[i][2] + b.z);
-      z[i][3] = tanhf(z[i][3] + b.w);
-      *(float4 *)(net.h1 + (row0 + r) * H + col) = make_float4(z[i][0], z[i][1], z[i][2], z[i][3]);
-      store_a<H>(a, kb, r, l16 * 4, z[i]);
+      for (int i = 0; i < 4; ++i) {
+        const int r = warp * kWR16 + i0 + 2 * i + rh;
+        *(float4 *)(net.h1 + (row0 + r) * H + col) = make_float4(z[i][0], z[i][1], z[i][2], z[i][3]);
+        store_a(a, r, l16 * 4, z[i]);
+      }
     }
     tc::fence_async_smem();
     tc::fence_before_sync();
     __syncwarp();
-    if (lane == 0) arrive(bars->a + kb);
+    if (lane == 0) arrive(&bars->a);
   }
+  float xn[XV];
+  if (next >= 0) load_x(d, rw, next, in, xn);
   // ---- layer 2's accumulator, then tanh and the output layer
-  const bool ok = call(tc::mbar_wait(&bars->acc, ph_acc, tc::kDrainNs));
+  const bool ok = call(tc::mbar_wait(&bars->acc, ph_acc, tc::kDrainNs) && okw);
   if (!ok) return false;
   tc::fence_after_sync();
   float *ct = (float *)reg;  // the operand tiles are free: every product has completed
@@ -155,10 +175,10 @@ __device__ __forceinline__ bool fwd_tile(const Net &net, Bars *bars, uint8_t *re
     csync();
     constexpr int LPR = G::CTW / 4, RPW = 32 / LPR;  // lanes per row, rows per warp access
     const int c = (lane % LPR) * 4;
-    const float4 b = __ldg((const float4 *)(net.b2 + c0 + c));
+    const float4 b = *(const float4 *)(net.b2 + c0 + c);
 #pragma unroll 2
-    for (int i = 0; i < 8; i += RPW) {
-      const int r = warp * 8 + i + lane / LPR;
+    for (int i = 0; i < kWR16; i += RPW) {
+      const int r = warp * kWR16 + i + lane / LPR;
       float4 v = *(float4 *)(ct + r * G::CP + c);
       v.x = tanhf(v.x + b.x);
       v.y = tanhf(v.y + b.y);
@@ -172,25 +192,26 @@ __device__ __forceinline__ bool fwd_tile(const Net &net, Bars *bars, uint8_t *re
       out_pass<H, (OUT > 0 ? OUT : 1)>(ct, net.W3, c0, acc);
     }
   }
+  if (next >= 0) store_x(xn, xp, xs);
   csync();  // ct is free
   if (OUT > 0) {
-    // the four unit groups' sums of a row, added in order
-    float *sp = ct;  // [4][128][OUT]
+    // the two unit groups' sums of a row
+    float *sp = ct;  // [2][128][OUT]
 #pragma unroll
     for (int o = 0; o < OUT; ++o) sp[tid * OUT + o] = acc[o];
     csync();
     for (int i = tid; i < kRows * OUT; i += kCT) {
       constexpr int P = kRows * (OUT > 0 ? OUT : 1);
-      net.out[row0 * OUT + i] = ((sp[i] + sp[P + i]) + (sp[2 * P + i] + sp[3 * P + i])) + __ldg(net.b3 + i % (OUT > 0 ? OUT : 1));
+      net.out[row0 * OUT + i] = (sp[i] + sp[P + i]) + __ldg(net.b3 + i % (OUT > 0 ? OUT : 1));
     }
     csync();
   }
   return true;
 }
 
-template <int H, int OUT>
-__global__ void __launch_bounds__(kThreads, 1)
-    k_train_fwd(Dev d, Rows rw, int in, int xp, const __grid_constant__ Nets nets) {
+template <int H, int OUT, int XV>
+__global__ void __launch_bounds__(kThreads, 2)
+    k_train_fwd(Dev d, Rows rw, int in, int xp, int off_w, const __grid_constant__ Nets nets) {
   using G = Geo<H>;
   using S = FwdSmem<H>;
   extern __shared__ uint8_t smem_raw[];
@@ -198,9 +219,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint8_t *sm = smem_raw + ((1024u - (raw & 1023u)) & 1023u);
   Bars *bars = (Bars *)(sm + S::OFF_BAR);
   float *xs = (float *)(sm + S::OFF_X);
+  float *ws = off_w ? (float *)(sm + off_w) : nullptr;
   const int tid = threadIdx.x, warp = tid >> 5;
   if (tid == 0) bars_init(bars);
-  if (warp == kCW) tc::tmem_alloc(&bars->tmem, H < 64 ? 64 : H);
+  if (warp == kCW) tc::tmem_alloc(&bars->tmem, H);
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
@@ -222,22 +244,39 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     __syncwarp();
   } else {
-    uint32_t ph = 0;
-    for (int q = 0; q < nets.count && ok; ++q)
-      for (int t = 0; t < my_tiles(tiles, q) && ok; ++t) {
+    uint32_t ph = 0, ph_af = 0;
+    for (int q = 0; q < nets.count && ok; ++q) {
+      Net net = nets.n[q];
+      const int mine = my_tiles(tiles, q), out = q == 0 ? OUT : 1;
+      if (mine == 0) continue;
+      float xn[XV];
+      load_x(d, rw, first_tile(tiles, q), in, xn);
+      csync();  // the last network's weights and observations are read
+      if (ws) {
+        for (int i = tid; i < (in + 1) * H; i += kCT) ws[i] = __ldg(net.W1 + i);
+        for (int i = tid; i < H; i += kCT) ws[(in + 1) * H + i] = __ldg(net.b2 + i);
+        for (int i = tid; i < out * H; i += kCT) ws[(in + 2) * H + i] = __ldg(net.W3 + i);
+        net.W1 = ws;
+        net.b1 = ws + in * H;
+        net.b2 = ws + (in + 1) * H;
+        net.W3 = ws + (in + 2) * H;
+      }
+      store_x(xn, xp, xs);
+      csync();
+      for (int t = 0; t < mine && ok; ++t) {
         const int tile = first_tile(tiles, q) + t * (int)gridDim.x;
-        gather_x(d, rw, tile, in, xp, xs);
-        csync();
-        ok = q == 0 ? fwd_tile<H, OUT>(nets.n[0], bars, sm, xs, in, xp, tile, tmem, ph)
-                    : fwd_tile<H, 1>(nets.n[1], bars, sm, xs, in, xp, tile, tmem, ph);
+        const int next = t + 1 < mine ? tile + (int)gridDim.x : -1;
+        ok = q == 0 ? fwd_tile<H, OUT, XV>(net, bars, sm, xs, in, xp, tile, tmem, ph, ph_af, d, rw, next)
+                    : fwd_tile<H, 1, XV>(net, bars, sm, xs, in, xp, tile, tmem, ph, ph_af, d, rw, next);
         ph ^= 1u;
       }
+    }
   }
   tc::fence_before_sync();
   __syncthreads();
   if (warp == kCW) {
     tc::fence_after_sync();
-    tc::tmem_dealloc(tmem, H < 64 ? 64 : H);
+    tc::tmem_dealloc(tmem, H);
   }
 }
 
@@ -248,14 +287,21 @@ int sm_count() {
   return sms;
 }
 
+template <int H, int OUT, int XV>
+cudaError_t run_fwd_x(const Dev &d, const Rows &rw, int in, const Nets &nets, cudaStream_t st) {
+  const int xp = (in + 3) & ~3, out = OUT > 1 ? OUT : 1, smem = FwdSmem<H>::bytes(in, xp, out);
+  const int off_w = FwdSmem<H>::w_fits(in, xp, out) ? FwdSmem<H>::off_w(xp) : 0;
+  cudaError_t e = cudaFuncSetAttribute(k_train_fwd<H, OUT, XV>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  const int tiles = nets.count * (int)((rw.rows + kRows - 1) / kRows), ctas = 2 * sm_count();
+  k_train_fwd<H, OUT, XV><<<tiles < ctas ? tiles : ctas, kThreads, smem, st>>>(d, rw, in, xp, off_w, nets);
+  return cudaGetLastError();
+}
 template <int H, int OUT>
 cudaError_t run_fwd(const Dev &d, const Rows &rw, int in, const Nets &nets, cudaStream_t st) {
-  const int xp = (in + 3) & ~3, smem = FwdSmem<H>::bytes(xp);
-  cudaError_t e = cudaFuncSetAttribute(k_train_fwd<H, OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
-  const int tiles = nets.count * (int)((rw.rows + kRows - 1) / kRows), sms = sm_count();
-  k_train_fwd<H, OUT><<<tiles < sms ? tiles : sms, kThreads, smem, st>>>(d, rw, in, xp, nets);
-  return cudaGetLastError();
+  if (in <= 2 * kXT) return run_fwd_x<H, OUT, 2>(d, rw, in, nets, st);
+  if (in <= 8 * kXT) return run_fwd_x<H, OUT, 8>(d, rw, in, nets, st);
+  return run_fwd_x<H, OUT, 12>(d, rw, in, nets, st);
 }
 
 template <int H>
