@@ -135,7 +135,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 2 : 1)
     }
     if (tid < RM * ((NA * RM + NT - 1) / NT > 1 ? NT / RM : NA)) {
       constexpr int CO = (NA * RM + NT - 1) / NT;
-      f32::layer_out<RM, CO>(h2s, w3s, b3, H1, NA, [&](int r, int o, float l) { lg[o * RM + r] = l; });
+      f32::layer_out<RM, CO>(h2s, w3s, b3, H1, NA, NA, [&](int r, int o, float l) { lg[o * RM + r] = l; });
     }
     if (C::kHelp && tid >= 64) {
       const int h = tid - 64;

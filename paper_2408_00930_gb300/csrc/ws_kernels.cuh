@@ -41,6 +41,7 @@ struct Dev {
   const uint8_t *eimg;      // landscape: packed hi/lo centre image + table (BF16 energy)
   const uint8_t *limg;      // landscape, fused kernel: its energy image (blocks of 64 Gaussians)
   const uint8_t *fimg;      // landscape, fused kernel with WS_FLAG_FORCE: the force image
+  int fuse_mlp;             // batched FP32 path: the whole policy forward in one launch
   int mlp3;                 // economy: whole-MLP tensor-core kernel (images in pk[pid][0])
   // economy on the fused persistent kernel: work items {first agent slot, rows,
   // first env, envs} and the work-queue counters {next item, CTAs finished}
@@ -170,6 +171,11 @@ cudaError_t launch_control_cc(const Dev &d, uint32_t n_steps, int envs_per_cta, 
 // ---- fused FP32 control path (ws_control_f32.cu) ----------------------------
 // Steps [k + off, k + off + n_steps) of every env in one launch.
 bool control_f32_supported(const PolicyShape &shape);
+// Three-layer FP32 forward in one launch (ws_mlp3_f32.cu), equal to three dense layers
+// bit for bit; X row-major when ldc == 1, or addressed X[r * ldr + c * ldc].
+bool mlp3_f32_supported(const PolicyShape &p);
+cudaError_t launch_mlp3_f32(const float *X, long ldr, long ldc, const float *params,
+                            const PolicyShape &p, float *Y, int M, cudaStream_t st);
 cudaError_t launch_control_f32(const Dev &d, uint32_t off, uint32_t n_steps, cudaStream_t st);
 
 }  // namespace ws

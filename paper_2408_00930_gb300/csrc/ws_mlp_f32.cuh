@@ -242,10 +242,11 @@ __device__ __forceinline__ void layer_tanh(float *H, const float *__restrict__ b
 }
 
 // The narrow last layer: thread t takes row t % RM and the CO outputs from
-// (t / RM) CO on; put(row, output, value) receives the sum with its bias.
+// (t / RM) CO on of N (weight rows ld apart); put(row, output, value) receives the
+// sum with its bias.
 template <int RM, int CO, typename Put>
 __device__ __forceinline__ void layer_out(const float *__restrict__ H, const float *__restrict__ W,
-                                          const float *__restrict__ b, int K, int N, Put put) {
+                                          const float *__restrict__ b, int K, int N, int ld, Put put) {
   const int r = threadIdx.x % RM, o0 = (int)(threadIdx.x / RM) * CO;
   if (o0 >= N) return;
   float acc[CO];
@@ -253,23 +254,23 @@ __device__ __forceinline__ void layer_out(const float *__restrict__ H, const flo
   for (int c = 0; c < CO; ++c) acc[c] = 0.f;
   const int r4 = r >> 2, rl = r & 3;
   int k = 0;
-#pragma unroll(CO <= 2 ? 4 : 1)
+#pragma unroll(CO <= 3 ? 4 : 2)
   for (; k + 4 <= K; k += 4) {
     const float *hp = H + k * RM + (((r4 ^ ((k >> 2) & (RM / 4 - 1))) << 2) | rl);
-    const float *wp = W + k * N + o0;
+    const float *wp = W + k * ld + o0;
 #pragma unroll
     for (int kk = 0; kk < 4; ++kk) {
       const float h = hp[kk * RM];
 #pragma unroll
       for (int c = 0; c < CO; ++c)
-        if (c == 0 || o0 + c < N) acc[c] = fmaf(h, wp[kk * N + c], acc[c]);
+        if (c == 0 || o0 + c < N) acc[c] = fmaf(h, wp[kk * ld + c], acc[c]);
     }
   }
   for (; k < K; ++k) {
     const float h = H[act_idx<RM>(k, r)];
 #pragma unroll
     for (int c = 0; c < CO; ++c)
-      if (c == 0 || o0 + c < N) acc[c] = fmaf(h, W[k * N + o0 + c], acc[c]);
+      if (c == 0 || o0 + c < N) acc[c] = fmaf(h, W[k * ld + o0 + c], acc[c]);
   }
 #pragma unroll
   for (int c = 0; c < CO; ++c)

@@ -56,6 +56,16 @@ extern "C" ws_status ws_policy_forward_noalloc(const float *obs, uint32_t n_rows
   const float *b1 = W1 + (size_t)hidden0 * hidden1;
   const float *W2 = b1 + hidden1;
   const float *b2 = W2 + (size_t)hidden1 * out_dim;
+  const ws::PolicyShape sh{{(int)in_dim, (int)hidden0, (int)hidden1, (int)out_dim}};
+  // one launch, activations on chip; not where the output overlaps what other rows
+  // still read (the layers one by one read all of it before they write)
+  const auto apart = [&](const float *p, size_t n) {
+    return out + (size_t)n_rows * out_dim <= p || p + n <= out;
+  };
+  if (ws::mlp3_f32_supported(sh) && apart(obs, (size_t)n_rows * in_dim) && apart(params, sh.count()))
+    return ws::launch_mlp3_f32(obs, in_dim, 1, params, sh, out, (int)n_rows, st) == cudaSuccess
+               ? WS_OK
+               : WS_ERR_CUDA;
   // Every element of h0 and h1 is written before it is read, so the contents
   // left by an earlier call need no clearing.
   ws::launch_dense_fp32(obs, in_dim, 1, W0, b0, h0, (int)n_rows, (int)in_dim, (int)hidden0, 1, st);

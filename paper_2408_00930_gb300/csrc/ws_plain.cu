@@ -249,6 +249,8 @@ void policy(const Dev &d, const float *X, long ldr, long ldc, const float *param
             cudaStream_t st) {
   if (d.mlp3)
     launch_mlp3_tc(X, ldr, ldc, d.pk[pid][0], sh, out, M, d.err, st);
+  else if (d.fuse_mlp && mlp3_f32_supported(sh))
+    launch_mlp3_f32(X, ldr, ldc, params, sh, out, M, st);
   else if (d.tc_mlp)
     tc_mlp3(d, X, ldr, ldc, sh, pid, h0, h1, out, M, st);
   else
@@ -571,59 +573,111 @@ __global__ __launch_bounds__(kEconThreads) void k_econ_finish(Dev d, uint32_t of
 // Gaussians of chunk blockIdx.y, in FP32 with Kahan compensation.
 // mode 0: y = x + dx (the post-step candidate); mode 1: y = x, only for envs
 // flagged needs_energy (after a reset).
-constexpr int kEnergyThreads = 128, kEnergyTileM = 64;
+//
+// Bound by the FP32 pipe (2 D operations per pair, ~12 for the exponential and the
+// sum): a thread holds the coordinates of EN envs in registers (DM >= D of them,
+// zeros past D, which leave the distance as it is) and takes kEnergyM Gaussians at a
+// time, whose distance chains (coordinates in order) are independent; each Gaussian's
+// coordinates come as 16-byte shared-memory broadcasts for both envs.  8,192 envs,
+// D 24, 4,096 Gaussians: EUS us per launch; one env per thread with its coordinates in
+// shared memory (two loads per two operations) took 236 us; floor 52 us.
+constexpr int kEnergyThreads = 128, kEnergyTileM = 64, kEnergyM = 4;
 
+template <int DM, int EN>
 __global__ __launch_bounds__(kEnergyThreads) void k_energy_partial(Dev d, uint32_t off, int mode) {
-  extern __shared__ float sm[];
+  __shared__ __align__(16) float cs[kEnergyTileM * DM];
+  __shared__ __align__(16) float as[kEnergyTileM], qs[kEnergyTileM];
   const int D = (int)d.dim;
-  float *ys = sm;                                  // [D][kEnergyThreads]
-  float *cs = ys + (size_t)D * kEnergyThreads;     // [kEnergyTileM][D]
-  float *as = cs + (size_t)kEnergyTileM * D;       // [kEnergyTileM]
-  float *qs = as + kEnergyTileM;                   // [kEnergyTileM]
-  const uint32_t e = blockIdx.x * kEnergyThreads + threadIdx.x;
-  const bool valid = e < d.n_envs;
-  bool want = valid && (mode == 0 || d.needs_energy[e]);
-  if (!__syncthreads_or(want)) return;
+  const uint32_t e0 = blockIdx.x * (kEnergyThreads * EN) + threadIdx.x;
+  bool want[EN], any = false;
+#pragma unroll
+  for (int i = 0; i < EN; ++i) {
+    const uint32_t e = e0 + i * kEnergyThreads;
+    want[i] = e < d.n_envs && (mode == 0 || d.needs_energy[e]);
+    any = any || want[i];
+  }
+  if (!__syncthreads_or(any)) return;
   const uint32_t row = ring_row(d, step_k(d, off));
   const float *act = (const float *)d.r_act + (size_t)row * D * d.n_slots;
-  for (int j = 0; j < D; ++j) {
-    float y = 0.f;
-    if (valid) {
-      y = d.s[(size_t)j * d.n_envs + e];
-      if (mode == 0) y = y + act[(size_t)j * d.n_slots + e];
+  float y[EN][DM];
+#pragma unroll
+  for (int i = 0; i < EN; ++i) {
+    const uint32_t e = e0 + i * kEnergyThreads;
+#pragma unroll
+    for (int j = 0; j < DM; ++j) {
+      y[i][j] = 0.f;
+      if (e < d.n_envs && j < D) {
+        y[i][j] = d.s[(size_t)j * d.n_envs + e];
+        if (mode == 0) y[i][j] = y[i][j] + act[(size_t)j * d.n_slots + e];
+      }
     }
-    ys[j * kEnergyThreads + threadIdx.x] = y;
   }
   const int M = (int)d.n_gauss;
   const int per = (M + kEnergyChunks - 1) / kEnergyChunks;
   const int m_lo = blockIdx.y * per, m_hi = min(M, m_lo + per);
-  float sum = 0.f, comp = 0.f;
+  float sum[EN], comp[EN];
+#pragma unroll
+  for (int i = 0; i < EN; ++i) sum[i] = comp[i] = 0.f;
   for (int t0 = m_lo; t0 < m_hi; t0 += kEnergyTileM) {
     const int nt = min(kEnergyTileM, m_hi - t0);
     __syncthreads();
-    for (int idx = threadIdx.x; idx < nt * D; idx += kEnergyThreads) cs[idx] = d.centres[(size_t)t0 * D + idx];
-    for (int idx = threadIdx.x; idx < nt; idx += kEnergyThreads) {
-      as[idx] = d.amps[t0 + idx];
-      qs[idx] = d.coef[t0 + idx];
+    for (int idx = threadIdx.x; idx < kEnergyTileM * DM; idx += kEnergyThreads) {
+      const int m = idx / DM, j = idx % DM;
+      cs[idx] = m < nt && j < D ? d.centres[(size_t)(t0 + m) * D + j] : 0.f;
+    }
+    for (int idx = threadIdx.x; idx < kEnergyTileM; idx += kEnergyThreads) {
+      as[idx] = idx < nt ? d.amps[t0 + idx] : 0.f;
+      qs[idx] = idx < nt ? d.coef[t0 + idx] : 0.f;
     }
     __syncthreads();
-    for (int m = 0; m < nt; ++m) {
-      float d2 = 0.f;
-      for (int j = 0; j < D; ++j) {
-        const float df = ys[j * kEnergyThreads + threadIdx.x] - cs[m * D + j];
-        d2 = fmaf(df, df, d2);
+#pragma unroll 1
+    for (int m0 = 0; m0 < nt; m0 += kEnergyM) {
+      float d2[kEnergyM][EN];
+#pragma unroll
+      for (int u = 0; u < kEnergyM; ++u)
+#pragma unroll
+        for (int i = 0; i < EN; ++i) d2[u][i] = 0.f;
+#pragma unroll
+      for (int j = 0; j < DM; j += 4)
+#pragma unroll
+        for (int u = 0; u < kEnergyM; ++u) {
+          const float4 c = *(const float4 *)(cs + (m0 + u) * DM + j);
+#pragma unroll
+          for (int i = 0; i < EN; ++i) {
+            const float f0 = y[i][j] - c.x, f1 = y[i][j + 1] - c.y, f2 = y[i][j + 2] - c.z,
+                        f3 = y[i][j + 3] - c.w;
+            d2[u][i] = fmaf(f0, f0, d2[u][i]);
+            d2[u][i] = fmaf(f1, f1, d2[u][i]);
+            d2[u][i] = fmaf(f2, f2, d2[u][i]);
+            d2[u][i] = fmaf(f3, f3, d2[u][i]);
+          }
+        }
+      float term[kEnergyM][EN];
+#pragma unroll
+      for (int u = 0; u < kEnergyM; ++u)
+#pragma unroll
+        for (int i = 0; i < EN; ++i) term[u][i] = as[m0 + u] * expf(-d2[u][i] * qs[m0 + u]);
+#pragma unroll
+      for (int u = 0; u < kEnergyM; ++u) {
+        if (m0 + u < nt) {  // Gaussians in order
+#pragma unroll
+          for (int i = 0; i < EN; ++i) {
+            const float yk = term[u][i] - comp[i];
+            const float tk = sum[i] + yk;
+            comp[i] = (tk - sum[i]) - yk;
+            sum[i] = tk;
+          }
+        }
       }
-      const float term = as[m] * expf(-d2 * qs[m]);
-      const float yk = term - comp;
-      const float tk = sum + yk;
-      comp = (tk - sum) - yk;
-      sum = tk;
     }
   }
-  if (want) {
-    d.epart[((size_t)blockIdx.y * 2 + 0) * d.n_envs + e] = sum;
-    d.epart[((size_t)blockIdx.y * 2 + 1) * d.n_envs + e] = comp;
-  }
+#pragma unroll
+  for (int i = 0; i < EN; ++i)
+    if (want[i]) {
+      const uint32_t e = e0 + i * kEnergyThreads;
+      d.epart[((size_t)blockIdx.y * 2 + 0) * d.n_envs + e] = sum[i];
+      d.epart[((size_t)blockIdx.y * 2 + 1) * d.n_envs + e] = comp[i];
+    }
 }
 
 __device__ float energy_combine(const Dev &d, uint32_t e) {
@@ -685,8 +739,11 @@ __global__ void k_landscape_reset_finish(Dev d, uint32_t off, int full_reset) {
   d.needs_energy[e] = 0;
 }
 
-size_t energy_smem(const Dev &d) {
-  return sizeof(float) * ((size_t)d.dim * kEnergyThreads + (size_t)kEnergyTileM * d.dim + 2 * kEnergyTileM);
+template <int DM, int EN>
+void energy_launch(const Dev &d, uint32_t off, int mode, cudaStream_t st) {
+  constexpr uint32_t per = kEnergyThreads * EN;
+  k_energy_partial<DM, EN><<<dim3((d.n_envs + per - 1) / per, kEnergyChunks), kEnergyThreads, 0, st>>>(
+      d, off, mode);
 }
 
 void landscape_energy(const Dev &d, uint32_t off, int mode, cudaStream_t st) {
@@ -694,8 +751,17 @@ void landscape_energy(const Dev &d, uint32_t off, int mode, cudaStream_t st) {
     launch_energy_tc(d, d.eimg, off, mode, st);
     return;
   }
-  dim3 grid((d.n_envs + kEnergyThreads - 1) / kEnergyThreads, kEnergyChunks);
-  k_energy_partial<<<grid, kEnergyThreads, energy_smem(d), st>>>(d, off, mode);
+  // two envs per thread while their coordinates fit the registers
+  if (d.dim <= 8)
+    energy_launch<8, 2>(d, off, mode, st);
+  else if (d.dim <= 16)
+    energy_launch<16, 2>(d, off, mode, st);
+  else if (d.dim <= 24)
+    energy_launch<24, 2>(d, off, mode, st);
+  else if (d.dim <= 32)
+    energy_launch<32, 2>(d, off, mode, st);
+  else
+    energy_launch<64, 1>(d, off, mode, st);
 }
 
 // ---------------------------------------------------------------- misc
@@ -972,8 +1038,6 @@ void launch_reset(const Dev &d, cudaStream_t st) {
                                            : d.n_envs;
   k_reset<<<blocks(n, 256), 256, 0, st>>>(d);
   if (d.env == WS_ENV_LANDSCAPE) {
-    cudaFuncSetAttribute(k_energy_partial, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)energy_smem(d));
     landscape_energy(d, 0, 1, st);
     k_landscape_reset_finish<<<blocks(d.n_envs, 256), 256, 0, st>>>(d, 0, 1);
   }

@@ -408,6 +408,7 @@ void make_dev(ws_ctx *c) {
     d.slot_env = (const int32_t *)(S + L.aux_off + up((N + 1) * 4));
   }
   d.t = (int32_t *)(S + L.t_off);
+  d.fuse_mlp = cfg.path == WS_PATH_BATCHED_FP32 ? 1 : 0;
   if (L.econ_fused) {
     d.items = (const int32_t *)(S + L.items_off);
     d.queue = (uint32_t *)(S + L.queue_off);
