@@ -79,6 +79,29 @@ __device__ __forceinline__ float2 box_muller(uint32_t w0, uint32_t w1) {
   return make_float2(rho * c, rho * s);
 }
 
+// Packed FP32 pairs (two operations per instruction, each lane rounded as the scalar
+// one): the FP32 pipe's rate is the same, the issue slots are half.
+__device__ __forceinline__ uint64_t f2_pack(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ float2 f2_unpack(uint64_t v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+
 WS_HD uint32_t bounded(uint32_t w, uint32_t n) { return mul_hi32(w, n); }
 
 // ------------------------------------------------------------------------

@@ -6,7 +6,8 @@
 // (ws_mlp_f32.cuh); every output is k_dense_fp32's chain, equal bit for bit.  Three
 // k_dense_fp32 launches passed each activation through memory and ran 16-deep stages
 // with two barriers each: 300 rows of 16-128-128-20 51 us, 8,192 rows of 4-256-256-2
-// 115 us, 8,192 rows of 24-256-256-48 116 us; here LS, LL and LN us.
+// 115 us, 8,192 rows of 24-256-256-48 116 us; here 10, 38 and
+// 60 us (floors 4, 14 and 18: the FP32 pipe, for the first the chain of phases).
 #include "ws_kernels.cuh"
 #include "ws_mlp_f32.cuh"
 
@@ -48,8 +49,11 @@ __device__ __forceinline__ void out_layer(const float *H, const float *__restric
     } else if (per <= 3) {
       f32::layer_out<RM, 3>(H, Wb, bb, K, left, N, put_b);
       base = N;
-    } else if (per <= 6) {
-      f32::layer_out<RM, 6>(H, Wb, bb, K, left, N, put_b);
+    } else if (per <= 4) {
+      f32::layer_out<RM, 4>(H, Wb, bb, K, left, N, put_b);
+      base = N;
+    } else if (per <= 8) {
+      f32::layer_out<RM, 8>(H, Wb, bb, K, left, N, put_b);
       base = N;
     } else {
       const int take = left < 12 * G ? left : 12 * G;

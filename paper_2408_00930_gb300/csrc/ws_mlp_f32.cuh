@@ -254,16 +254,38 @@ __device__ __forceinline__ void layer_out(const float *__restrict__ H, const flo
   for (int c = 0; c < CO; ++c) acc[c] = 0.f;
   const int r4 = r >> 2, rl = r & 3;
   int k = 0;
+  // 16-byte weight loads where every row's share starts on 16 bytes and is whole
+  const bool vec = CO % 4 == 0 && (ld & 3) == 0 && ((uintptr_t)W & 15) == 0 && o0 + CO <= N;
+  if (vec) {
+#pragma unroll 2
+    for (; k + 4 <= K; k += 4) {
+      const float *hp = H + k * RM + (((r4 ^ ((k >> 2) & (RM / 4 - 1))) << 2) | rl);
+      const float *wp = W + k * ld + o0;
+#pragma unroll
+      for (int kk = 0; kk < 4; ++kk) {
+        const float h = hp[kk * RM];
+#pragma unroll
+        for (int c = 0; c + 4 <= CO; c += 4) {
+          const float4 w = *(const float4 *)(wp + kk * ld + c);
+          acc[c] = fmaf(h, w.x, acc[c]);
+          acc[c + 1] = fmaf(h, w.y, acc[c + 1]);
+          acc[c + 2] = fmaf(h, w.z, acc[c + 2]);
+          acc[c + 3] = fmaf(h, w.w, acc[c + 3]);
+        }
+      }
+    }
+  } else {
 #pragma unroll(CO <= 3 ? 4 : 2)
-  for (; k + 4 <= K; k += 4) {
-    const float *hp = H + k * RM + (((r4 ^ ((k >> 2) & (RM / 4 - 1))) << 2) | rl);
-    const float *wp = W + k * ld + o0;
+    for (; k + 4 <= K; k += 4) {
+      const float *hp = H + k * RM + (((r4 ^ ((k >> 2) & (RM / 4 - 1))) << 2) | rl);
+      const float *wp = W + k * ld + o0;
 #pragma unroll
-    for (int kk = 0; kk < 4; ++kk) {
-      const float h = hp[kk * RM];
+      for (int kk = 0; kk < 4; ++kk) {
+        const float h = hp[kk * RM];
 #pragma unroll
-      for (int c = 0; c < CO; ++c)
-        if (c == 0 || o0 + c < N) acc[c] = fmaf(h, wp[kk * ld + c], acc[c]);
+        for (int c = 0; c < CO; ++c)
+          if (c == 0 || o0 + c < N) acc[c] = fmaf(h, wp[kk * ld + c], acc[c]);
+      }
     }
   }
   for (; k < K; ++k) {

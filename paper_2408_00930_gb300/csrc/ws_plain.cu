@@ -575,109 +575,105 @@ __global__ __launch_bounds__(kEconThreads) void k_econ_finish(Dev d, uint32_t of
 // flagged needs_energy (after a reset).
 //
 // Bound by the FP32 pipe (2 D operations per pair, ~12 for the exponential and the
-// sum): a thread holds the coordinates of EN envs in registers (DM >= D of them,
-// zeros past D, which leave the distance as it is) and takes kEnergyM Gaussians at a
-// time, whose distance chains (coordinates in order) are independent; each Gaussian's
-// coordinates come as 16-byte shared-memory broadcasts for both envs.  8,192 envs,
-// D 24, 4,096 Gaussians: EUS us per launch; one env per thread with its coordinates in
-// shared memory (two loads per two operations) took 236 us; floor 52 us.
-constexpr int kEnergyThreads = 128, kEnergyTileM = 64, kEnergyM = 4;
+// sum): a thread holds its env's coordinates in registers, doubled (DM >= D of them,
+// zeros past D, which leave the distance as it is), and takes kEnergyM Gaussians at a
+// time in pairs, the two lanes of packed operations, whose distance chains
+// (coordinates in order) are independent; the pair's coordinates come interleaved and
+// negated as 16-byte shared-memory broadcasts, the next tile's loads in flight.  8,192
+// envs, D 24, 4,096 Gaussians: 86 us per launch (floor 52); coordinates in shared
+// memory, two loads per two operations: 236; two envs per thread: 94 (half the warps).
+constexpr int kEnergyThreads = 128, kEnergyTileM = 64, kEnergyM = 8;
 
-template <int DM, int EN>
+template <int DM>
 __global__ __launch_bounds__(kEnergyThreads) void k_energy_partial(Dev d, uint32_t off, int mode) {
-  __shared__ __align__(16) float cs[kEnergyTileM * DM];
-  __shared__ __align__(16) float as[kEnergyTileM], qs[kEnergyTileM];
+  __shared__ __align__(16) float cs[kEnergyTileM / 2 * DM * 2];  // [pair][j]{-c_m, -c_m+1}
+  __shared__ float as[kEnergyTileM], qs[kEnergyTileM];
   const int D = (int)d.dim;
-  const uint32_t e0 = blockIdx.x * (kEnergyThreads * EN) + threadIdx.x;
-  bool want[EN], any = false;
-#pragma unroll
-  for (int i = 0; i < EN; ++i) {
-    const uint32_t e = e0 + i * kEnergyThreads;
-    want[i] = e < d.n_envs && (mode == 0 || d.needs_energy[e]);
-    any = any || want[i];
-  }
-  if (!__syncthreads_or(any)) return;
+  const uint32_t e = blockIdx.x * kEnergyThreads + threadIdx.x;
+  const bool want = e < d.n_envs && (mode == 0 || d.needs_energy[e]);
+  if (!__syncthreads_or(want)) return;
   const uint32_t row = ring_row(d, step_k(d, off));
   const float *act = (const float *)d.r_act + (size_t)row * D * d.n_slots;
-  float y[EN][DM];
+  uint64_t y[DM];
 #pragma unroll
-  for (int i = 0; i < EN; ++i) {
-    const uint32_t e = e0 + i * kEnergyThreads;
-#pragma unroll
-    for (int j = 0; j < DM; ++j) {
-      y[i][j] = 0.f;
-      if (e < d.n_envs && j < D) {
-        y[i][j] = d.s[(size_t)j * d.n_envs + e];
-        if (mode == 0) y[i][j] = y[i][j] + act[(size_t)j * d.n_slots + e];
-      }
+  for (int j = 0; j < DM; ++j) {
+    float x = 0.f;
+    if (e < d.n_envs && j < D) {
+      x = d.s[(size_t)j * d.n_envs + e];
+      if (mode == 0) x = x + act[(size_t)j * d.n_slots + e];
     }
+    y[j] = f2_pack(x, x);
   }
   const int M = (int)d.n_gauss;
   const int per = (M + kEnergyChunks - 1) / kEnergyChunks;
   const int m_lo = blockIdx.y * per, m_hi = min(M, m_lo + per);
-  float sum[EN], comp[EN];
+  // the next tile in registers: thread t takes elements t, t + 128, ... of [m][DM]
+  constexpr int NV = kEnergyTileM * DM / kEnergyThreads;
+  float nv[NV], na = 0.f, nq = 0.f;
+  auto fetch = [&](int t0) {
+    const int nt = min(kEnergyTileM, m_hi - t0);
 #pragma unroll
-  for (int i = 0; i < EN; ++i) sum[i] = comp[i] = 0.f;
+    for (int v = 0; v < NV; ++v) {
+      const int idx = threadIdx.x + v * kEnergyThreads, m = idx / DM, j = idx % DM;
+      nv[v] = m < nt && j < D ? __ldg(d.centres + (size_t)(t0 + m) * D + j) : 0.f;
+    }
+    if (threadIdx.x < kEnergyTileM) {
+      const bool in = (int)threadIdx.x < nt;
+      na = in ? __ldg(d.amps + t0 + threadIdx.x) : 0.f;
+      nq = in ? __ldg(d.coef + t0 + threadIdx.x) : 0.f;
+    }
+  };
+  float sum = 0.f, comp = 0.f;
+  if (m_lo < m_hi) fetch(m_lo);
   for (int t0 = m_lo; t0 < m_hi; t0 += kEnergyTileM) {
     const int nt = min(kEnergyTileM, m_hi - t0);
     __syncthreads();
-    for (int idx = threadIdx.x; idx < kEnergyTileM * DM; idx += kEnergyThreads) {
-      const int m = idx / DM, j = idx % DM;
-      cs[idx] = m < nt && j < D ? d.centres[(size_t)(t0 + m) * D + j] : 0.f;
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      const int idx = threadIdx.x + v * kEnergyThreads, m = idx / DM, j = idx % DM;
+      cs[((m >> 1) * DM + j) * 2 + (m & 1)] = -nv[v];
     }
-    for (int idx = threadIdx.x; idx < kEnergyTileM; idx += kEnergyThreads) {
-      as[idx] = idx < nt ? d.amps[t0 + idx] : 0.f;
-      qs[idx] = idx < nt ? d.coef[t0 + idx] : 0.f;
+    if (threadIdx.x < kEnergyTileM) {
+      as[threadIdx.x] = na;
+      qs[threadIdx.x] = nq;
     }
     __syncthreads();
+    if (t0 + kEnergyTileM < m_hi) fetch(t0 + kEnergyTileM);
 #pragma unroll 1
     for (int m0 = 0; m0 < nt; m0 += kEnergyM) {
-      float d2[kEnergyM][EN];
+      uint64_t d2[kEnergyM / 2];
 #pragma unroll
-      for (int u = 0; u < kEnergyM; ++u)
+      for (int u = 0; u < kEnergyM / 2; ++u) d2[u] = 0ull;
 #pragma unroll
-        for (int i = 0; i < EN; ++i) d2[u][i] = 0.f;
+      for (int j = 0; j < DM; j += 2)
 #pragma unroll
-      for (int j = 0; j < DM; j += 4)
-#pragma unroll
-        for (int u = 0; u < kEnergyM; ++u) {
-          const float4 c = *(const float4 *)(cs + (m0 + u) * DM + j);
-#pragma unroll
-          for (int i = 0; i < EN; ++i) {
-            const float f0 = y[i][j] - c.x, f1 = y[i][j + 1] - c.y, f2 = y[i][j + 2] - c.z,
-                        f3 = y[i][j + 3] - c.w;
-            d2[u][i] = fmaf(f0, f0, d2[u][i]);
-            d2[u][i] = fmaf(f1, f1, d2[u][i]);
-            d2[u][i] = fmaf(f2, f2, d2[u][i]);
-            d2[u][i] = fmaf(f3, f3, d2[u][i]);
-          }
+        for (int u = 0; u < kEnergyM / 2; ++u) {
+          const ulonglong2 c = *(const ulonglong2 *)(cs + ((m0 / 2 + u) * DM + j) * 2);
+          const uint64_t f0 = f2_add(y[j], c.x), f1 = f2_add(y[j + 1], c.y);
+          d2[u] = f2_fma(f0, f0, d2[u]);
+          d2[u] = f2_fma(f1, f1, d2[u]);
         }
-      float term[kEnergyM][EN];
+      float term[kEnergyM];
 #pragma unroll
-      for (int u = 0; u < kEnergyM; ++u)
-#pragma unroll
-        for (int i = 0; i < EN; ++i) term[u][i] = as[m0 + u] * expf(-d2[u][i] * qs[m0 + u]);
+      for (int u = 0; u < kEnergyM; ++u) {
+        const float2 q = f2_unpack(d2[u / 2]);
+        term[u] = as[m0 + u] * expf(-((u & 1) ? q.y : q.x) * qs[m0 + u]);
+      }
 #pragma unroll
       for (int u = 0; u < kEnergyM; ++u) {
         if (m0 + u < nt) {  // Gaussians in order
-#pragma unroll
-          for (int i = 0; i < EN; ++i) {
-            const float yk = term[u][i] - comp[i];
-            const float tk = sum[i] + yk;
-            comp[i] = (tk - sum[i]) - yk;
-            sum[i] = tk;
-          }
+          const float yk = term[u] - comp;
+          const float tk = sum + yk;
+          comp = (tk - sum) - yk;
+          sum = tk;
         }
       }
     }
   }
-#pragma unroll
-  for (int i = 0; i < EN; ++i)
-    if (want[i]) {
-      const uint32_t e = e0 + i * kEnergyThreads;
-      d.epart[((size_t)blockIdx.y * 2 + 0) * d.n_envs + e] = sum[i];
-      d.epart[((size_t)blockIdx.y * 2 + 1) * d.n_envs + e] = comp[i];
-    }
+  if (want) {
+    d.epart[((size_t)blockIdx.y * 2 + 0) * d.n_envs + e] = sum;
+    d.epart[((size_t)blockIdx.y * 2 + 1) * d.n_envs + e] = comp;
+  }
 }
 
 __device__ float energy_combine(const Dev &d, uint32_t e) {
@@ -739,11 +735,10 @@ __global__ void k_landscape_reset_finish(Dev d, uint32_t off, int full_reset) {
   d.needs_energy[e] = 0;
 }
 
-template <int DM, int EN>
+template <int DM>
 void energy_launch(const Dev &d, uint32_t off, int mode, cudaStream_t st) {
-  constexpr uint32_t per = kEnergyThreads * EN;
-  k_energy_partial<DM, EN><<<dim3((d.n_envs + per - 1) / per, kEnergyChunks), kEnergyThreads, 0, st>>>(
-      d, off, mode);
+  k_energy_partial<DM><<<dim3((d.n_envs + kEnergyThreads - 1) / kEnergyThreads, kEnergyChunks),
+                         kEnergyThreads, 0, st>>>(d, off, mode);
 }
 
 void landscape_energy(const Dev &d, uint32_t off, int mode, cudaStream_t st) {
@@ -751,17 +746,16 @@ void landscape_energy(const Dev &d, uint32_t off, int mode, cudaStream_t st) {
     launch_energy_tc(d, d.eimg, off, mode, st);
     return;
   }
-  // two envs per thread while their coordinates fit the registers
   if (d.dim <= 8)
-    energy_launch<8, 2>(d, off, mode, st);
+    energy_launch<8>(d, off, mode, st);
   else if (d.dim <= 16)
-    energy_launch<16, 2>(d, off, mode, st);
+    energy_launch<16>(d, off, mode, st);
   else if (d.dim <= 24)
-    energy_launch<24, 2>(d, off, mode, st);
+    energy_launch<24>(d, off, mode, st);
   else if (d.dim <= 32)
-    energy_launch<32, 2>(d, off, mode, st);
+    energy_launch<32>(d, off, mode, st);
   else
-    energy_launch<64, 1>(d, off, mode, st);
+    energy_launch<64>(d, off, mode, st);
 }
 
 // ---------------------------------------------------------------- misc
