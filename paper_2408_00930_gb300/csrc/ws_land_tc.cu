@@ -943,35 +943,39 @@ __global__ void __launch_bounds__(kRollThreads, 1)
 // F(y) = -grad E(y) = sum_m s_m P_m (y - c_m) / w_m^2 with P_m = |a_m| e_m and
 // s_m the sign of a_m:
 //   F_j = y_j * sum_m P_m f_m  -  sum_m P_m f_m c_mj,   f_m = s_m / w_m^2.
-// Per 128-row tile of (step, env) rows: each 64-Gaussian block's whole
+// Per 128-row tile of (step, env) rows: each 128-Gaussian block's whole
 // exponents log2 P_m come from the energy image exactly as in the roll-out
-// sweep (one MMA, K = 80, into one of four TMEM accumulators); the epilogue
-// turns them into P = 2^z (one ex2 per pair) and writes P as BF16 hi + lo into
-// a shared-memory A operand [128 rows][64 Gaussians]; a second MMA multiplies
-// it with the block's force image [32 columns][64 Gaussians] = (f c_m, f, 0...)
-// (hi + lo; three products hi.hi + lo.hi + hi.lo) into one FP32 accumulator of
-// 32 columns per row.  The sign and 1 / w^2 ride in the force image, so the
-// epilogue is the exponential and the split alone.
+// sweep (K = 80, N = 128, the operand rows in tensor memory, into one of three
+// 128-column accumulators); the epilogue turns them into P = 2^z (one ex2 per pair)
+// and writes P as BF16 hi + lo back over the accumulator's own columns, where it is
+// the A operand of the force product; that multiplies it with the block's force
+// image [64 columns][128 Gaussians] = (f c_m, f, 0...) hi beside lo (three products
+// hi.hi, hi.lo in one N = 64 instruction, lo.hi in an N = 32 one) into FP32
+// accumulators of 2 x 32 columns per row.  The sign and 1 / w^2 ride in the force
+// image, so the epilogue is the exponential and the split alone.
+//
+// Bound by the tensor pipe's instructions: 21 per 128 Gaussians here.  Over 64-Gaussian
+// blocks with P through shared memory it was 34 (at ~115 cycles each, every one
+// reading 4 KB of A from shared memory): 1.436 ms for 8,192 envs x 50 steps x 4,096
+// Gaussians, D 24; now FTUS ms.  The epilogue's ex2 floor is 0.17 ms.
 constexpr int kFN = 32;                          // force columns: D coordinates, the sum, zeros
 constexpr int kFImgBytes = kFN * kBlk * 2;       // one plane of a block's force image
 constexpr int kFBlkBytes = 2 * kFImgBytes;       // hi plane | lo plane
-constexpr int kFS = 4;                           // shared-memory stages (energy + force block)
-constexpr int kFStage = kBlkBytes + kFBlkBytes;
-constexpr int kFZ = 4;                           // TMEM exponent accumulators
-constexpr int kFP = 3;                           // P operand buffers
-constexpr int kPPlane = kRows * kBlk * 2;        // one plane of P [128][64]
-constexpr uint32_t TM_F = kFZ * kBlk;            // TMEM columns of the force accumulator
-constexpr int FOFF_AE = 0;
-constexpr int FOFF_ST = FOFF_AE + kRows * kKE * 2;
-constexpr int FOFF_P = FOFF_ST + kFS * kFStage;
-constexpr int FOFF_BAR = FOFF_P + kFP * 2 * kPPlane;
-constexpr int F_NBAR = 1 + 2 * kFS + 2 * kFZ + 2 * kFP + 2;  // ae, b, sf, z, zf, p, pf, f, drain
+constexpr int kFS = 5;                           // shared-memory stages (energy + force, kEB Gaussians)
+constexpr int kFStage = 2 * (kBlkBytes + kFBlkBytes);
+constexpr int kFZ = 3;                           // TMEM exponent accumulators, then P operands
+constexpr int kFLook = 2;                        // blocks the exponents run ahead of the force
+constexpr uint32_t TM_F = kFZ * kEB;             // TMEM columns of the force accumulators
+constexpr uint32_t TM_FA = TM_F + 2 * kFN;       // TMEM columns of the operand rows
+constexpr int FOFF_ST = 0;
+constexpr int FOFF_BAR = FOFF_ST + kFS * kFStage;
+constexpr int F_NBAR = 1 + 2 * kFS + 3 * kFZ + 2;  // ae, b, sf, z, p, pf, f, drain
 constexpr int FOFF_CMD = FOFF_BAR + F_NBAR * 8;
 constexpr int FOFF_TM = FOFF_CMD + 16;
 constexpr int FSMEM = FOFF_TM + 16 + 1024;
 static_assert(FSMEM <= 232448, "force kernel shared memory");
-static_assert(FOFF_ST % 16 == 0 && FOFF_P % 16 == 0 && FOFF_BAR % 8 == 0, "alignment");
-static_assert(TM_F + kFN <= 512, "force accumulator");
+static_assert(FOFF_ST % 16 == 0 && FOFF_BAR % 8 == 0, "alignment");
+static_assert(TM_FA + kKE / 2 <= 512, "accumulators and operand rows");
 
 inline size_t force_img_bytes(int M) { return (size_t)(land_slots(M) / kBlk) * kFBlkBytes; }
 
@@ -1006,8 +1010,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int tid = threadIdx.x, warp = tid >> 5;
   uint64_t *bars = (uint64_t *)(sm + FOFF_BAR);
   uint64_t *bar_ae = bars, *bar_b = bar_ae + 1, *bar_sf = bar_b + kFS, *bar_z = bar_sf + kFS;
-  uint64_t *bar_zf = bar_z + kFZ, *bar_p = bar_zf + kFZ, *bar_pf = bar_p + kFP;
-  uint64_t *bar_f = bar_pf + kFP, *bar_drain = bar_f + 1;
+  uint64_t *bar_p = bar_z + kFZ, *bar_pf = bar_p + kFZ, *bar_f = bar_pf + kFZ, *bar_drain = bar_f + 1;
   volatile uint32_t *cmd = (volatile uint32_t *)(sm + FOFF_CMD);
   uint32_t *tm_holder = (uint32_t *)(sm + FOFF_TM);
   if (tid == 0) {
@@ -1018,9 +1021,6 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     for (int i = 0; i < kFZ; ++i) {
       tc::mbar_init(bar_z + i, 1);
-      tc::mbar_init(bar_zf + i, kEpi);
-    }
-    for (int i = 0; i < kFP; ++i) {
       tc::mbar_init(bar_p + i, kEpi);
       tc::mbar_init(bar_pf + i, 1);
     }
@@ -1036,7 +1036,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const uint32_t tbase = *tm_holder;
   const size_t N = d.n_envs, S = d.n_slots, rows = (size_t)n * N;
   const int n_tiles = (int)((rows + kRows - 1) / kRows);
-  const int nb = ((const int32_t *)eimg)[0];  // blocks per tile (all Gaussians)
+  const int nb = ((const int32_t *)eimg)[0] / 2;  // kEB-Gaussian blocks per tile (all Gaussians)
   int my_tiles = 0;
   for (int t = (int)blockIdx.x; t < n_tiles; t += (int)gridDim.x) ++my_tiles;
   const uint32_t total = (uint32_t)my_tiles * (uint32_t)nb;
@@ -1045,9 +1045,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (tid >= kEpi) {
     // ===================== producer warps =====================
     // Block g (counted over this CTA's tiles) sits in stage g % kFS, its
-    // exponents in TMEM accumulator g % kFZ, its P in buffer g % kFP.  The MMA
-    // warp issues the exponent MMA of block g, then the force MMA of block g - 1,
-    // so the tensor core works on g while the epilogue exponentiates g - 1.
+    // exponents, then its P, in TMEM buffer g % kFZ.  The MMA warp issues the
+    // exponent MMAs of block g, then the force MMAs of block g - kFLook, so the
+    // tensor core works on g while the epilogue exponentiates the blocks between.
     const int lane = tid & 31;
     if (warp == kEpi / 32) {
       if (lane == 0) {
@@ -1056,11 +1056,11 @@ __global__ void __launch_bounds__(kThreads, 1)
           const uint32_t st = gl % kFS;
           if (gl >= (uint32_t)kFS &&
               !tc::mbar_wait(bar_sf + st, ((gl - kFS) / kFS) & 1u, kWaitNs)) { fail = true; break; }
-          const uint32_t b = gl % (uint32_t)nb;
+          const uint32_t b = 2u * (gl % (uint32_t)nb);
           mbar_expect_tx(bar_b + st, kFStage);
-          bulk_g2s(sb + FOFF_ST + st * kFStage, eblocks + (size_t)b * kBlkBytes, kBlkBytes, bar_b + st);
-          bulk_g2s(sb + FOFF_ST + st * kFStage + kBlkBytes, fblocks + (size_t)b * kFBlkBytes,
-                   kFBlkBytes, bar_b + st);
+          bulk_g2s(sb + FOFF_ST + st * kFStage, eblocks + (size_t)b * kBlkBytes, 2 * kBlkBytes, bar_b + st);
+          bulk_g2s(sb + FOFF_ST + st * kFStage + 2 * kBlkBytes, fblocks + (size_t)b * kFBlkBytes,
+                   2 * kFBlkBytes, bar_b + st);
         }
         cmd[0] = gl;
       }
@@ -1069,26 +1069,25 @@ __global__ void __launch_bounds__(kThreads, 1)
     } else {
       uint32_t g = 0;
       if (lane == 0) {
-        constexpr uint32_t id_e = tc::idesc_bf16_f32(128, kBlk), id_f = tc::idesc_bf16_f32(128, kFN);
-        // force MMA of block q: three products of P (hi, lo) and the image (hi, lo)
+        constexpr uint32_t id_e = tc::idesc_bf16_f32(128, kEB), id_f1 = tc::idesc_bf16_f32(128, kFN),
+                           id_f2 = tc::idesc_bf16_f32(128, 2 * kFN);
+        // force MMAs of block q: P_hi against the hi and lo planes (64 rows of B, the
+        // planes lie one after the other), P_lo against the hi plane
         auto force_mma = [&](uint32_t q, bool first) -> bool {
-          const uint32_t pb = q % kFP, st = q % kFS;
-          if (!tc::mbar_wait(bar_p + pb, (q / kFP) & 1u, kWaitNs)) return false;
+          const uint32_t z = q % kFZ, st = q % kFS;
+          if (!tc::mbar_wait(bar_p + z, (q / kFZ) & 1u, kWaitNs)) return false;
           tc::fence_after_sync();
-          const uint32_t pa = sb + FOFF_P + pb * 2u * kPPlane;
-          const uint32_t fb = sb + FOFF_ST + st * kFStage + kBlkBytes;
+          const uint32_t fb = sb + FOFF_ST + st * kFStage + 2 * kBlkBytes;
 #pragma unroll
-          for (int prod = 0; prod < 3; ++prod) {
-            const uint32_t a0 = pa + (prod == 1 ? (uint32_t)kPPlane : 0u);
-            const uint32_t b0 = fb + (prod == 2 ? (uint32_t)kFImgBytes : 0u);
-#pragma unroll
-            for (int s = 0; s < kBlk / 16; ++s) {
-              const uint64_t da = tc::smem_desc(a0 + (uint32_t)s * 256u, 128, kBlk * 16, tc::kSwizzleNone);
-              const uint64_t db = tc::smem_desc(b0 + (uint32_t)s * 256u, 128, kBlk * 16, tc::kSwizzleNone);
-              tc::mma_bf16(tbase + TM_F, da, db, id_f, !(first && prod == 0 && s == 0));
-            }
+          for (int s = 0; s < kEB / 16; ++s) {
+            // K step s: P_hi in columns 32 (s / 2) + 8 (s % 2).., P_lo 16 columns on
+            const uint32_t pa = tbase + z * kEB + (uint32_t)(32 * (s / 2) + 8 * (s % 2));
+            const uint64_t db = tc::smem_desc(fb + (uint32_t)(s / 4) * kFBlkBytes + (uint32_t)(s % 4) * 256u,
+                                              128, kBlk * 16, tc::kSwizzleNone);
+            mma_ts(tbase + TM_F, pa, db, id_f2, !(first && s == 0));
+            mma_ts(tbase + TM_F, pa + 16u, db, id_f1, true);
           }
-          tc::mma_commit(bar_pf + pb);
+          tc::mma_commit(bar_pf + z);
           tc::mma_commit(bar_sf + st);
           return true;
         };
@@ -1096,25 +1095,29 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int t = 0; t < my_tiles && !fail; ++t) {
           if (!tc::mbar_wait(bar_ae, pa, kWaitNs)) { fail = true; break; }
           pa ^= 1u;
-          for (int i = 0; i < nb; ++i, ++g) {
-            const uint32_t st = g % kFS, z = g % kFZ;
-            if (!tc::mbar_wait(bar_b + st, (g / kFS) & 1u, kWaitNs)) { fail = true; break; }
-            if (g >= (uint32_t)kFZ &&
-                !tc::mbar_wait(bar_zf + z, ((g - kFZ) / kFZ) & 1u, kWaitNs)) { fail = true; break; }
-            tc::fence_after_sync();
+          for (int i = 0; i < nb + kFLook; ++i) {
+            if (i < nb) {
+              const uint32_t st = g % kFS, z = g % kFZ;
+              if (!tc::mbar_wait(bar_b + st, (g / kFS) & 1u, kWaitNs)) { fail = true; break; }
+              if (g >= (uint32_t)kFZ &&
+                  !tc::mbar_wait(bar_pf + z, ((g - kFZ) / kFZ) & 1u, kWaitNs)) { fail = true; break; }
+              tc::fence_after_sync();
 #pragma unroll
-            for (int s = 0; s < kKE / 16; ++s) {
-              const uint64_t da = tc::smem_desc(sb + FOFF_AE + (uint32_t)s * 256u, 128, kKE * 16,
-                                                tc::kSwizzleNone);
-              const uint64_t db = tc::smem_desc(sb + FOFF_ST + st * kFStage + (uint32_t)s * 256u, 128,
-                                                kKE * 16, tc::kSwizzleNone);
-              tc::mma_bf16(tbase + z * kBlk, da, db, id_e, s != 0);
+              for (int s = 0; s < kKE / 16; ++s) {
+                const uint64_t db = tc::smem_desc(sb + FOFF_ST + st * kFStage + (uint32_t)s * 256u, 128,
+                                                  kKE * 16, tc::kSwizzleNone);
+                mma_ts(tbase + z * kEB, tbase + TM_FA + (uint32_t)(8 * s), db, id_e, s != 0);
+              }
+              tc::mma_commit(bar_z + z);
+              ++g;
             }
-            tc::mma_commit(bar_z + z);
-            if (i > 0 && !force_mma(g - 1, i == 1)) { fail = true; break; }
+            if (i >= kFLook) {
+              // block i - kFLook of the tile
+              const uint32_t q = g - (uint32_t)(i < nb ? kFLook + 1 : nb + kFLook - i);
+              if (!force_mma(q, i == kFLook)) { fail = true; break; }
+            }
           }
           if (fail) break;
-          if (!force_mma(g - 1, nb == 1)) { fail = true; break; }
           tc::mma_commit(bar_f);
         }
       }
@@ -1137,12 +1140,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   } else {
     // ===================== epilogue =====================
     // Row r of a tile: thread r (half 0) holds y, writes the operand row and the
-    // force; threads r and r + 128 exponentiate columns [32 h, 32 h + 32) of
+    // force; threads r and r + 128 exponentiate columns [64 h, 64 h + 64) of
     // every block.
     const int r = tid & 127, h = tid >> 7;
     const uint32_t lane_sel = (uint32_t)((warp & 3) * 32) << 16;
-    const uint32_t ae_row = sb + FOFF_AE + (uint32_t)(r >> 3) * (kKE * 16) + (uint32_t)(r & 7) * 16u;
-    auto kofs = [](int k) -> uint32_t { return (uint32_t)((k >> 3) * 128 + (k & 7) * 2); };
     const uint64_t k_end = d.k[0];
     uint32_t g = 0, pf = 0;
     for (int tile = (int)blockIdx.x; tile < n_tiles && !fail; tile += (int)gridDim.x) {
@@ -1160,75 +1161,78 @@ __global__ void __launch_bounds__(kThreads, 1)
           y[j] = valid ? obs[(size_t)j * S] + act[(size_t)j * S] : 0.f;
           yy = fmaf(y[j], y[j], yy);
         }
-        // [y_hi | y_hi | y_lo | 1, 1 | yy_hi, yy_hi, yy_lo | 0...]
+        // [y_hi | y_hi | y_lo | 1, 1 | yy_hi, yy_hi, yy_lo | 0...], two per column
+        uint32_t hw[D / 2], lw[D / 2];
 #pragma unroll
-        for (int q4 = 0; q4 < D / 4; ++q4) {
-          const float a0 = y[4 * q4], a1 = y[4 * q4 + 1], a2 = y[4 * q4 + 2], a3 = y[4 * q4 + 3];
-          const uint32_t h01 = tc::pack_bf16x2(a0, a1), h23 = tc::pack_bf16x2(a2, a3);
-          const uint32_t l01 = tc::pack_bf16x2(a0 - tc::bf16_lo(h01), a1 - tc::bf16_hi(h01));
-          const uint32_t l23 = tc::pack_bf16x2(a2 - tc::bf16_lo(h23), a3 - tc::bf16_hi(h23));
-          const int j = 4 * q4;
-          asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(ae_row + kofs(j)), "r"(h01), "r"(h23) : "memory");
-          asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(ae_row + kofs(D + j)), "r"(h01), "r"(h23) : "memory");
-          asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(ae_row + kofs(2 * D + j)), "r"(l01), "r"(l23) : "memory");
+        for (int c = 0; c < D / 2; ++c) {
+          hw[c] = tc::pack_bf16x2(y[2 * c], y[2 * c + 1]);
+          lw[c] = tc::pack_bf16x2(y[2 * c] - tc::bf16_lo(hw[c]), y[2 * c + 1] - tc::bf16_hi(hw[c]));
         }
         const uint32_t hv = tc::pack_bf16x2(yy, 0.f) & 0xFFFFu;
         const uint32_t lv = tc::pack_bf16x2(yy - __uint_as_float(hv << 16), 0.f) & 0xFFFFu;
+        constexpr int NT = kKE / 2 - 3 * D / 2;
+        uint32_t tw[NT];
 #pragma unroll
-        for (int c = 3 * D / 8; c < kKE / 8; ++c) {
-          if (c == 3 * D / 8)
-            tc::sts128(ae_row + (uint32_t)c * 128u, tc::pack_bf16x2(1.f, 1.f), hv | (hv << 16), lv, 0u);
-          else
-            tc::sts128(ae_row + (uint32_t)c * 128u, 0u, 0u, 0u, 0u);
-        }
-        tc::fence_async_smem();
+        for (int c = 0; c < NT; ++c) tw[c] = 0u;
+        tw[0] = tc::pack_bf16x2(1.f, 1.f);
+        tw[1] = hv | (hv << 16);
+        tw[2] = lv;
+        const uint32_t ae = tbase + lane_sel + TM_FA;
+        tmem_st_cols<D / 2>(ae, hw);
+        tmem_st_cols<D / 2>(ae + (uint32_t)(D / 2), hw);
+        tmem_st_cols<D / 2>(ae + (uint32_t)D, lw);
+        tmem_st_cols<NT>(ae + (uint32_t)(3 * D / 2), tw);
+        tmem_wait_st();
+        tc::fence_before_sync();
         mbar_arrive(bar_ae);
       }
-      // ---- the blocks: P = 2^z as BF16 hi + lo into the A operand of the force MMA
-      const uint32_t p_row = (uint32_t)(r >> 3) * (kBlk * 16) + (uint32_t)(r & 7) * 16u;
+      // ---- the blocks: P = 2^z as BF16 hi + lo over the exponents, 32 columns at a
+      // time: the hi pairs in the first 16, the lo pairs in the other 16
       for (int b = 0; b < nb; ++b, ++g) {
-        const uint32_t z = g % kFZ, pb = g % kFP;
+        const uint32_t z = g % kFZ;
         if (!tc::mbar_wait(bar_z + z, (g / kFZ) & 1u, kWaitNs)) { fail = true; break; }
         tc::fence_after_sync();
-        uint32_t v[32];
-        tc::tmem_ld32(tbase + lane_sel + z * kBlk + (uint32_t)(32 * h), v);
-        tc::tmem_wait_ld();
-        tc::fence_before_sync();
-        mbar_arrive(bar_zf + z);
-        if (g >= (uint32_t)kFP &&
-            !tc::mbar_wait(bar_pf + pb, ((g - kFP) / kFP) & 1u, kWaitNs)) { fail = true; break; }
-        const uint32_t pbase = sb + FOFF_P + pb * 2u * kPPlane + p_row;
+        const uint32_t col = tbase + lane_sel + z * kEB + (uint32_t)(64 * h);
+        uint32_t v0[32], v1[32];
+        tc::tmem_ld32(col, v0);
+        tc::tmem_ld32(col + 32u, v1);
+        tmem_wait_ld_regs(v0);
+        tmem_wait_ld_regs(v1);
+        auto split = [](const uint32_t (&v)[32], uint32_t (&o)[32]) {
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          uint32_t hi[4], lo[4];
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const float p0 = ex2_fast(__uint_as_float(v[8 * c + 2 * u]));
-            const float p1 = ex2_fast(__uint_as_float(v[8 * c + 2 * u + 1]));
-            hi[u] = tc::pack_bf16x2(p0, p1);
-            lo[u] = tc::pack_bf16x2(p0 - tc::bf16_lo(hi[u]), p1 - tc::bf16_hi(hi[u]));
+          for (int c = 0; c < 16; ++c) {
+            const float p0 = ex2_fast(__uint_as_float(v[2 * c])), p1 = ex2_fast(__uint_as_float(v[2 * c + 1]));
+            o[c] = tc::pack_bf16x2(p0, p1);
+            o[16 + c] = tc::pack_bf16x2(p0 - tc::bf16_lo(o[c]), p1 - tc::bf16_hi(o[c]));
           }
-          const uint32_t off = (uint32_t)((4 * h + c) * 128);
-          tc::sts128(pbase + off, hi[0], hi[1], hi[2], hi[3]);
-          tc::sts128(pbase + kPPlane + off, lo[0], lo[1], lo[2], lo[3]);
-        }
-        tc::fence_async_smem();
-        mbar_arrive(bar_p + pb);
+        };
+        uint32_t o[32];
+        split(v0, o);
+        tmem_st32(col, o);
+        split(v1, o);
+        tmem_st32(col + 32u, o);
+        tmem_wait_st();
+        tc::fence_before_sync();
+        mbar_arrive(bar_p + z);
       }
       if (fail) break;
       // ---- the tile's force: F_j = y_j * acc[D] - acc[j]
       if (h == 0) {
         if (!tc::mbar_wait(bar_f, pf, kWaitNs)) { fail = true; break; }
         tc::fence_after_sync();
-        uint32_t acc[32];
+        uint32_t acc[32], acl[32];
         tc::tmem_ld32(tbase + lane_sel + TM_F, acc);
-        tc::tmem_wait_ld();
+        tc::tmem_ld32(tbase + lane_sel + TM_F + kFN, acl);
+        tmem_wait_ld_regs(acc);
+        tmem_wait_ld_regs(acl);
         tc::fence_before_sync();
         if (valid) {
-          const float sp = __uint_as_float(acc[D]);
+          const float sp = __uint_as_float(acc[D]) + __uint_as_float(acl[D]);
           float *out = d.r_force + rowR * D * S + e;
 #pragma unroll
-          for (int j = 0; j < D; ++j) out[(size_t)j * S] = fmaf(y[j], sp, -__uint_as_float(acc[j]));
+          for (int j = 0; j < D; ++j)
+            out[(size_t)j * S] =
+                fmaf(y[j], sp, -(__uint_as_float(acc[j]) + __uint_as_float(acl[j])));
         }
       }
       pf ^= 1u;
