@@ -957,21 +957,21 @@ __global__ void __launch_bounds__(kRollThreads, 1)
 // Bound by the tensor pipe's instructions: 21 per 128 Gaussians here.  Over 64-Gaussian
 // blocks with P through shared memory it was 34 (at ~115 cycles each, every one
 // reading 4 KB of A from shared memory): 1.436 ms for 8,192 envs x 50 steps x 4,096
-// Gaussians, D 24; now FTUS ms.  The epilogue's ex2 floor is 0.17 ms.
+// Gaussians, D 24; now 0.70 ms (0.92 with one warp issuing both
+// products, 0.86 with the halves on alternate blocks).  The epilogue's ex2 floor is 0.17 ms.
+constexpr int kForceThreads = kEpi + 96;         // + a loader warp and two MMA warps
 constexpr int kFN = 32;                          // force columns: D coordinates, the sum, zeros
 constexpr int kFImgBytes = kFN * kBlk * 2;       // one plane of a block's force image
 constexpr int kFBlkBytes = 2 * kFImgBytes;       // hi plane | lo plane
 constexpr int kFS = 5;                           // shared-memory stages (energy + force, kEB Gaussians)
 constexpr int kFStage = 2 * (kBlkBytes + kFBlkBytes);
 constexpr int kFZ = 3;                           // TMEM exponent accumulators, then P operands
-constexpr int kFLook = 2;                        // blocks the exponents run ahead of the force
 constexpr uint32_t TM_F = kFZ * kEB;             // TMEM columns of the force accumulators
 constexpr uint32_t TM_FA = TM_F + 2 * kFN;       // TMEM columns of the operand rows
 constexpr int FOFF_ST = 0;
 constexpr int FOFF_BAR = FOFF_ST + kFS * kFStage;
 constexpr int F_NBAR = 1 + 2 * kFS + 3 * kFZ + 2;  // ae, b, sf, z, p, pf, f, drain
-constexpr int FOFF_CMD = FOFF_BAR + F_NBAR * 8;
-constexpr int FOFF_TM = FOFF_CMD + 16;
+constexpr int FOFF_TM = FOFF_BAR + (F_NBAR + 1) / 2 * 16;
 constexpr int FSMEM = FOFF_TM + 16 + 1024;
 static_assert(FSMEM <= 232448, "force kernel shared memory");
 static_assert(FOFF_ST % 16 == 0 && FOFF_BAR % 8 == 0, "alignment");
@@ -1000,7 +1000,7 @@ __global__ void k_force_tc_pack(const float *__restrict__ c, const float *__rest
 }
 
 template <int D>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kForceThreads, 1)
     k_force_tc(Dev d, const uint8_t *__restrict__ eimg, const uint8_t *__restrict__ eblocks,
                const uint8_t *__restrict__ fblocks, uint32_t n) {
   extern __shared__ uint8_t smem_raw[];
@@ -1011,7 +1011,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint64_t *bars = (uint64_t *)(sm + FOFF_BAR);
   uint64_t *bar_ae = bars, *bar_b = bar_ae + 1, *bar_sf = bar_b + kFS, *bar_z = bar_sf + kFS;
   uint64_t *bar_p = bar_z + kFZ, *bar_pf = bar_p + kFZ, *bar_f = bar_pf + kFZ, *bar_drain = bar_f + 1;
-  volatile uint32_t *cmd = (volatile uint32_t *)(sm + FOFF_CMD);
   uint32_t *tm_holder = (uint32_t *)(sm + FOFF_TM);
   if (tid == 0) {
     tc::mbar_init(bar_ae, kRows);  // half 0 writes the operand rows
@@ -1021,12 +1020,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     for (int i = 0; i < kFZ; ++i) {
       tc::mbar_init(bar_z + i, 1);
-      tc::mbar_init(bar_p + i, kEpi);
+      tc::mbar_init(bar_p + i, kRows);  // the half that exponentiates the block
       tc::mbar_init(bar_pf + i, 1);
     }
     tc::mbar_init(bar_f, 1);
-    tc::mbar_init(bar_drain, 1);
-    cmd[0] = 0u;
+    tc::mbar_init(bar_drain, 2);  // both MMA warps
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) tc::tmem_alloc(tm_holder, 512);
@@ -1045,13 +1043,13 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (tid >= kEpi) {
     // ===================== producer warps =====================
     // Block g (counted over this CTA's tiles) sits in stage g % kFS, its
-    // exponents, then its P, in TMEM buffer g % kFZ.  The MMA warp issues the
-    // exponent MMAs of block g, then the force MMAs of block g - kFLook, so the
-    // tensor core works on g while the epilogue exponentiates the blocks between.
+    // exponents, then its P, in TMEM buffer g % kFZ.  One warp loads, one issues the
+    // exponent MMAs and one the force MMAs: an issuing thread is held for about as long
+    // as its instructions run, so the two sequences and their waits overlap.
     const int lane = tid & 31;
+    uint32_t gl = 0;
     if (warp == kEpi / 32) {
       if (lane == 0) {
-        uint32_t gl = 0;
         for (; gl < total && !fail; ++gl) {
           const uint32_t st = gl % kFS;
           if (gl >= (uint32_t)kFS &&
@@ -1062,76 +1060,73 @@ __global__ void __launch_bounds__(kThreads, 1)
           bulk_g2s(sb + FOFF_ST + st * kFStage + 2 * kBlkBytes, fblocks + (size_t)b * kFBlkBytes,
                    2 * kFBlkBytes, bar_b + st);
         }
-        cmd[0] = gl;
+        // copies issued ahead of a wait that ran out (here or in another warp) land
+        // before shared memory goes away
+        for (uint32_t q = gl > (uint32_t)kFS ? gl - kFS : 0u; q < gl; ++q)
+          tc::mbar_wait(bar_b + q % kFS, (q / kFS) & 1u, kWaitNs);
       }
       __syncwarp();
-      bar_sync_n(kBarProd, 64);
-    } else {
-      uint32_t g = 0;
+    } else if (warp == kEpi / 32 + 1) {
       if (lane == 0) {
-        constexpr uint32_t id_e = tc::idesc_bf16_f32(128, kEB), id_f1 = tc::idesc_bf16_f32(128, kFN),
-                           id_f2 = tc::idesc_bf16_f32(128, 2 * kFN);
-        // force MMAs of block q: P_hi against the hi and lo planes (64 rows of B, the
-        // planes lie one after the other), P_lo against the hi plane
-        auto force_mma = [&](uint32_t q, bool first) -> bool {
-          const uint32_t z = q % kFZ, st = q % kFS;
-          if (!tc::mbar_wait(bar_p + z, (q / kFZ) & 1u, kWaitNs)) return false;
-          tc::fence_after_sync();
-          const uint32_t fb = sb + FOFF_ST + st * kFStage + 2 * kBlkBytes;
-#pragma unroll
-          for (int s = 0; s < kEB / 16; ++s) {
-            // K step s: P_hi in columns 32 (s / 2) + 8 (s % 2).., P_lo 16 columns on
-            const uint32_t pa = tbase + z * kEB + (uint32_t)(32 * (s / 2) + 8 * (s % 2));
-            const uint64_t db = tc::smem_desc(fb + (uint32_t)(s / 4) * kFBlkBytes + (uint32_t)(s % 4) * 256u,
-                                              128, kBlk * 16, tc::kSwizzleNone);
-            mma_ts(tbase + TM_F, pa, db, id_f2, !(first && s == 0));
-            mma_ts(tbase + TM_F, pa + 16u, db, id_f1, true);
-          }
-          tc::mma_commit(bar_pf + z);
-          tc::mma_commit(bar_sf + st);
-          return true;
-        };
-        uint32_t pa = 0;
+        constexpr uint32_t id_e = tc::idesc_bf16_f32(128, kEB);
+        uint32_t g = 0, pa = 0;
         for (int t = 0; t < my_tiles && !fail; ++t) {
           if (!tc::mbar_wait(bar_ae, pa, kWaitNs)) { fail = true; break; }
           pa ^= 1u;
-          for (int i = 0; i < nb + kFLook; ++i) {
-            if (i < nb) {
-              const uint32_t st = g % kFS, z = g % kFZ;
-              if (!tc::mbar_wait(bar_b + st, (g / kFS) & 1u, kWaitNs)) { fail = true; break; }
-              if (g >= (uint32_t)kFZ &&
-                  !tc::mbar_wait(bar_pf + z, ((g - kFZ) / kFZ) & 1u, kWaitNs)) { fail = true; break; }
-              tc::fence_after_sync();
+          for (int i = 0; i < nb; ++i, ++g) {
+            const uint32_t st = g % kFS, z = g % kFZ;
+            if (!tc::mbar_wait(bar_b + st, (g / kFS) & 1u, kWaitNs)) { fail = true; break; }
+            if (g >= (uint32_t)kFZ &&
+                !tc::mbar_wait(bar_pf + z, ((g - kFZ) / kFZ) & 1u, kWaitNs)) { fail = true; break; }
+            tc::fence_after_sync();
 #pragma unroll
-              for (int s = 0; s < kKE / 16; ++s) {
-                const uint64_t db = tc::smem_desc(sb + FOFF_ST + st * kFStage + (uint32_t)s * 256u, 128,
-                                                  kKE * 16, tc::kSwizzleNone);
-                mma_ts(tbase + z * kEB, tbase + TM_FA + (uint32_t)(8 * s), db, id_e, s != 0);
-              }
-              tc::mma_commit(bar_z + z);
-              ++g;
+            for (int s = 0; s < kKE / 16; ++s) {
+              const uint64_t db = tc::smem_desc(sb + FOFF_ST + st * kFStage + (uint32_t)s * 256u, 128,
+                                                kKE * 16, tc::kSwizzleNone);
+              mma_ts(tbase + z * kEB, tbase + TM_FA + (uint32_t)(8 * s), db, id_e, s != 0);
             }
-            if (i >= kFLook) {
-              // block i - kFLook of the tile
-              const uint32_t q = g - (uint32_t)(i < nb ? kFLook + 1 : nb + kFLook - i);
-              if (!force_mma(q, i == kFLook)) { fail = true; break; }
-            }
+            tc::mma_commit(bar_z + z);
           }
-          if (fail) break;
-          tc::mma_commit(bar_f);
-        }
-      }
-      __syncwarp();
-      bar_sync_n(kBarProd, 64);
-      if (lane == 0) {
-        // copies issued ahead of a wait that ran out land before shared memory goes away
-        if (fail) {
-          const uint32_t gl = cmd[0];
-          for (uint32_t q = g; q < gl; ++q) tc::mbar_wait(bar_b + q % kFS, (q / kFS) & 1u, kWaitNs);
         }
         tc::mma_commit(bar_drain);
         tc::mbar_wait(bar_drain, 0, kWaitNs);
       }
+      __syncwarp();
+    } else {
+      if (lane == 0) {
+        // force MMAs: P_hi against the hi and lo planes (64 rows of B, the planes lie
+        // one after the other), P_lo against the hi plane
+        constexpr uint32_t id_f1 = tc::idesc_bf16_f32(128, kFN), id_f2 = tc::idesc_bf16_f32(128, 2 * kFN);
+        uint32_t g = 0;
+        for (int t = 0; t < my_tiles && !fail; ++t) {
+          for (int i = 0; i < nb; ++i, ++g) {
+            const uint32_t st = g % kFS, z = g % kFZ;
+            if (!tc::mbar_wait(bar_p + z, (g / kFZ) & 1u, kWaitNs)) { fail = true; break; }
+            // (the block's copies: waited on by the exponents' warp, and here for this
+            // thread's own view of them)
+            if (!tc::mbar_wait(bar_b + st, (g / kFS) & 1u, kWaitNs)) { fail = true; break; }
+            tc::fence_after_sync();
+            const uint32_t fb = sb + FOFF_ST + st * kFStage + 2 * kBlkBytes;
+#pragma unroll
+            for (int s = 0; s < kEB / 16; ++s) {
+              // K step s: P_hi in columns 32 (s / 2) + 8 (s % 2).., P_lo 16 columns on
+              const uint32_t pc = tbase + z * kEB + (uint32_t)(32 * (s / 2) + 8 * (s % 2));
+              const uint64_t db = tc::smem_desc(
+                  fb + (uint32_t)(s / 4) * kFBlkBytes + (uint32_t)(s % 4) * 256u, 128, kBlk * 16,
+                  tc::kSwizzleNone);
+              mma_ts(tbase + TM_F, pc, db, id_f2, !(i == 0 && s == 0));
+              mma_ts(tbase + TM_F, pc + 16u, db, id_f1, true);
+            }
+            tc::mma_commit(bar_pf + z);
+            tc::mma_commit(bar_sf + st);
+          }
+          if (fail) break;
+          tc::mma_commit(bar_f);
+        }
+        tc::mma_commit(bar_drain);
+        tc::mbar_wait(bar_drain, 0, kWaitNs);
+      }
+      __syncwarp();
     }
     if (fail && (tid & 31) == 0) {
       atomicExch(d.err, 1u);
@@ -1140,8 +1135,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   } else {
     // ===================== epilogue =====================
     // Row r of a tile: thread r (half 0) holds y, writes the operand row and the
-    // force; threads r and r + 128 exponentiate columns [64 h, 64 h + 64) of
-    // every block.
+    // force; threads r and r + 128 exponentiate the even and the odd blocks.
     const int r = tid & 127, h = tid >> 7;
     const uint32_t lane_sel = (uint32_t)((warp & 3) * 32) << 16;
     const uint64_t k_end = d.k[0];
@@ -1187,17 +1181,16 @@ __global__ void __launch_bounds__(kThreads, 1)
         mbar_arrive(bar_ae);
       }
       // ---- the blocks: P = 2^z as BF16 hi + lo over the exponents, 32 columns at a
-      // time: the hi pairs in the first 16, the lo pairs in the other 16
+      // time: the hi pairs in the first 16, the lo pairs in the other 16.  Half h
+      // takes every other block (by the CTA's running count), so that one block's
+      // waits and tensor-memory round trips run under the other's exponentials; the
+      // next chunk loads while one is worked on
       for (int b = 0; b < nb; ++b, ++g) {
+        if ((g & 1u) != (uint32_t)h) continue;
         const uint32_t z = g % kFZ;
         if (!tc::mbar_wait(bar_z + z, (g / kFZ) & 1u, kWaitNs)) { fail = true; break; }
         tc::fence_after_sync();
-        const uint32_t col = tbase + lane_sel + z * kEB + (uint32_t)(64 * h);
-        uint32_t v0[32], v1[32];
-        tc::tmem_ld32(col, v0);
-        tc::tmem_ld32(col + 32u, v1);
-        tmem_wait_ld_regs(v0);
-        tmem_wait_ld_regs(v1);
+        const uint32_t col = tbase + lane_sel + z * kEB;
         auto split = [](const uint32_t (&v)[32], uint32_t (&o)[32]) {
 #pragma unroll
           for (int c = 0; c < 16; ++c) {
@@ -1206,11 +1199,23 @@ __global__ void __launch_bounds__(kThreads, 1)
             o[16 + c] = tc::pack_bf16x2(p0 - tc::bf16_lo(o[c]), p1 - tc::bf16_hi(o[c]));
           }
         };
-        uint32_t o[32];
-        split(v0, o);
+        uint32_t va[32], vb[32], o[32];
+        tc::tmem_ld32(col, va);
+        tmem_wait_ld_regs(va);
+        tc::tmem_ld32(col + 32u, vb);
+        split(va, o);
         tmem_st32(col, o);
-        split(v1, o);
+        tmem_wait_ld_regs(vb);
+        tc::tmem_ld32(col + 64u, va);
+        split(vb, o);
         tmem_st32(col + 32u, o);
+        tmem_wait_ld_regs(va);
+        tc::tmem_ld32(col + 96u, vb);
+        split(va, o);
+        tmem_st32(col + 64u, o);
+        tmem_wait_ld_regs(vb);
+        split(vb, o);
+        tmem_st32(col + 96u, o);
         tmem_wait_st();
         tc::fence_before_sync();
         mbar_arrive(bar_p + z);
@@ -1264,7 +1269,7 @@ cudaError_t launch_force_d(const Dev &d, const uint8_t *eimg, const uint8_t *fim
   const size_t rows = (size_t)n * d.n_envs;
   const int n_tiles = (int)((rows + kRows - 1) / kRows);
   const int grid = n_tiles < sms ? n_tiles : sms;
-  k_force_tc<D><<<grid, kThreads, FSMEM, st>>>(d, eimg, eimg + land_blocks_off((int)d.n_gauss), fimg, n);
+  k_force_tc<D><<<grid, kForceThreads, FSMEM, st>>>(d, eimg, eimg + land_blocks_off((int)d.n_gauss), fimg, n);
   return cudaGetLastError();
 }
 
