@@ -64,3 +64,10 @@ def test_noalloc_forward_edges(rows, widths):
         got = out[:rows * widths[3]].cpu().numpy().reshape(rows, widths[3])
         err = np.abs(got - ref) / np.maximum(np.abs(ref).max(axis=1, keepdims=True), 1.0)
         assert err.max() <= TOL_F32
+
+
+@pytest.mark.parametrize("rows,widths", [
+    (1, (24, 128, 128, 48)), (9, (1, 65, 128, 33)), (1215, (16, 128, 37, 17)), (2432, (23, 100, 66, 32)),
+    (2431, (4, 64, 64, 16)), (8, (24, 33, 64, 48))])
+def test_noalloc_forward_few_rows(rows, widths):
+    test_noalloc_forward_edges(rows, widths)
