@@ -14,7 +14,7 @@
 // the env and writes the records.  W1, b3 and W3 stay in shared memory for the
 // launch; W2 too up to 128 units (64 KB), else its rows are streamed from L2.
 //
-// What bounds it: the FP32 FMA pipe for many envs (131,072 envs, 4-256-256-2: 380
+// What bounds it: the FP32 FMA pipe for many envs (131,072 envs, 4-256-256-2: 372
 // us per step against 1,003 us for the six kernels; 67% of the pipe's cycles busy
 // with the products' and tanhf's FMAs, floor 253 us), the step's own chain of
 // dependent phases for few (1,000 envs, 4-64-64-2: 1.2 us per step against 32 us).
@@ -181,7 +181,9 @@ struct Cfg {
   static constexpr bool kHelp = RM * E::NA <= 64 && 2 * RM <= 64;
 };
 
-template <typename E, int NT, int TM, int CPT, int ST>
+// PAD: H0 is no multiple of 4 (in the kernel of the other widths the test alone costs 3%
+// at 256 units: 391 against 378 us per step).
+template <typename E, int NT, int TM, int CPT, int ST, bool PAD>
 __global__ void __launch_bounds__(NT, NT == 256 ? 2 : 1)
     k_ctrl_f32(Dev d, uint32_t off, uint32_t n_steps) {
   using C = Cfg<E, NT, TM, CPT, ST>;
@@ -237,6 +239,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 2 : 1)
       uint64_t acc[TM][CPT / 2];
       f32::layer_product<NT, TM, CPT, 0>(xs, w1s, nullptr, OBS, H0, acc);
       f32::layer_tanh<NT, TM, CPT>(h1s, b1, H0, acc);
+      if (PAD) f32::zero_pad<NT, RM>(h1s, H0);
       f32::layer_product<NT, TM, CPT, ST>(h1s, ST == 0 ? w2s : W2, w2s, H0, H1, acc);
       f32::layer_tanh<NT, TM, CPT>(h2s, b2, H1, acc);
     }
@@ -340,6 +343,11 @@ __global__ void __launch_bounds__(128, HP == 64 ? 4 : 2)
     }
   };
   if (tid >= 64 && tid < 64 + 2 * RM) draws((uint32_t)k0, tid - 64, 0);
+  // units past H0 keep zeros (an infinite observation times their zero weights is NaN):
+  // their results go to the column past the units
+  const int uc = u < H0 ? u : HP;
+  if (u >= H0)
+    for (int r = 0; r < RPT; ++r) h1s[(r0 + r) * C::P + u] = 0.f;
   uint32_t row = (uint32_t)(k0 % R);
   for (uint32_t j = 0; j < n_steps; ++j) {
     const uint32_t k = (uint32_t)(k0 + j);
@@ -357,7 +365,7 @@ __global__ void __launch_bounds__(128, HP == 64 ? 4 : 2)
       float z = 0.f;
 #pragma unroll
       for (int i = 0; i < OBS; ++i) z = fmaf(xs[(r0 + r) * 8 + i], w1c[i], z);
-      h1s[(r0 + r) * C::P + u] = tanhf(z + b1u);
+      h1s[(r0 + r) * C::P + uc] = tanhf(z + b1u);
     }
     __syncthreads();
     // ---- layer 2
@@ -432,11 +440,11 @@ cudaError_t run_u(const Dev &d, uint32_t off, uint32_t n, cudaStream_t st) {
 template <typename E, int NT, int TM, int CPT, int ST>
 cudaError_t run(const Dev &d, uint32_t off, uint32_t n, cudaStream_t st) {
   using C = Cfg<E, NT, TM, CPT, ST>;
-  cudaError_t e = cudaFuncSetAttribute(k_ctrl_f32<E, NT, TM, CPT, ST>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
+  const auto kernel = (d.pol.w[1] & 3) ? k_ctrl_f32<E, NT, TM, CPT, ST, true>
+                                       : k_ctrl_f32<E, NT, TM, CPT, ST, false>;
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
   if (e != cudaSuccess) return e;
-  k_ctrl_f32<E, NT, TM, CPT, ST>
-      <<<(d.n_envs + C::RM - 1) / C::RM, NT, C::SMEM, st>>>(d, off, n);
+  kernel<<<(d.n_envs + C::RM - 1) / C::RM, NT, C::SMEM, st>>>(d, off, n);
   return cudaGetLastError();
 }
 

@@ -93,6 +93,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 2 : 1)
   uint64_t acc[TM][CPT / 2];
   f32::layer_product<NT, TM, CPT, ST>(xs, W0, st, w0, w1, acc);
   f32::layer_tanh<NT, TM, CPT>(h1s, b0, w1, acc);
+  f32::zero_pad<NT, C::RM>(h1s, w1);
   f32::layer_product<NT, TM, CPT, ST>(h1s, W1, st, w1, w2, acc);
   f32::layer_tanh<NT, TM, CPT>(h2s, b1, w2, acc);
   out_layer<NT, RM>(h2s, W2, b2, w2, w3, row0, M, Y);
@@ -146,6 +147,8 @@ __global__ void __launch_bounds__(128)
   float w0c[kUnitIn];
 #pragma unroll
   for (int k = 0; k < kUnitIn; ++k) w0c[k] = (u < w1 && k < w0) ? __ldg(W0 + k * w1 + u) : 0.f;
+  if (u >= w1)  // zeros past w1 (an infinite input times their zero weights is NaN)
+    for (int r = 0; r < RPT; ++r) h1s[(r0 + r) * P + u] = 0.f;
   const float b0u = u < w1 ? __ldg(b0 + u) : 0.f, b1u = u < w2 ? __ldg(b1 + u) : 0.f;
   for (int i = tid; i < RM * w0; i += NT) {
     const int r = i / w0, k = i % w0;
@@ -162,7 +165,7 @@ __global__ void __launch_bounds__(128)
 #pragma unroll
         for (int r = 0; r < RPT; ++r) z[r] = fmaf(xs[(r0 + r) * XP + k], w0c[k], z[r]);
 #pragma unroll
-    for (int r = 0; r < RPT; ++r) h1s[(r0 + r) * P + u] = tanhf(z[r] + b0u);
+    for (int r = 0; r < RPT; ++r) h1s[(r0 + r) * P + (u < w1 ? u : HP)] = tanhf(z[r] + b0u);
   }
   __syncthreads();
   {

@@ -186,12 +186,12 @@ __device__ __forceinline__ void layer_product(const float *A, const float *W, fl
   __syncthreads();  // the stages are free
 }
 
-// tanh(acc + b) into H (columns past N are tanh(0) = 0, the next layer's zero
-// padding).  Small tiles apply tanhf in registers; larger ones write the
-// pre-activations and apply it in place over the array (the unrolled tanhf of
-// 32 to 128 values per thread would not fit the instruction cache).  H may be the
-// product's own input when the tile is large (a CTA barrier separates them).
-// Ends with a CTA barrier.
+// tanh(acc + b) into H (columns past N are tanh(0) = 0, the next layer's zero padding;
+// zero_pad where an input may be infinite, which times a zero weight is NaN).  Small
+// tiles apply tanhf in registers; larger ones write the pre-activations and apply it in
+// place over the array (the unrolled tanhf of 32 to 128 values per thread would not fit
+// the instruction cache).  H may be the product's own input when the tile is large (a
+// CTA barrier separates them).  Ends with a CTA barrier.
 template <int NT, int TM, int CPT>
 __device__ __forceinline__ void layer_tanh(float *H, const float *__restrict__ b, int N,
                                            const uint64_t (&acc)[TM][CPT / 2]) {
@@ -239,6 +239,15 @@ __device__ __forceinline__ void layer_tanh(float *H, const float *__restrict__ b
     }
     __syncthreads();
   }
+}
+
+// Zeros in the columns from N to a multiple of 4, for every width that has such columns.
+template <int NT, int RM>
+__device__ __forceinline__ void zero_pad(float *H, int N) {
+  if ((N & 3) == 0) return;
+  const int n1 = N * (RM / 4), n4 = ((N + 3) & ~3) * (RM / 4);
+  if ((int)threadIdx.x < n4 - n1) ((float4 *)H)[n1 + threadIdx.x] = make_float4(0.f, 0.f, 0.f, 0.f);
+  __syncthreads();
 }
 
 // The narrow last layer: thread t takes row t % RM and the CO outputs from

@@ -34,3 +34,23 @@ def test_fused_fp32_equals_plain(env, h0, h1):
         b = _records(env, W.WS_PATH_BATCHED_FP32, n, T, h0, h1, ring)
         for i, (x, y) in enumerate(zip(a, b)):
             assert np.array_equal(x.view(np.uint8), y.view(np.uint8)), (n, i)
+
+
+@pytest.mark.parametrize("h0,h1", [(61, 33), (37, 100), (130, 253)])
+def test_infinite_state_stays_in_its_row(h0, h1):
+    # an infinite observation against a unit past the width (a zero weight) must not reach the units there are
+    for n in (77, 31000):
+        rows = []
+        for path in (W.WS_PATH_PLAIN_FP32, W.WS_PATH_BATCHED_FP32):
+            r = W.Rollout(W.WS_ENV_CONTROL, path, n, 4, 13, h0, h1, param_seed=3, flags=W.WS_FLAG_DEBUG_LOGITS)
+            r.reset(11)
+            state = r.fetch_raw(W.WS_F_STATE, 20 * n).copy()
+            state[:16 * n].view(np.float32).reshape(4, n)[0, 5] = np.inf
+            r.load_raw(W.WS_F_STATE, state, k=0)
+            r.rollout(4)
+            r.sync()
+            rows.append([r.fetch(f, 0, 4) for f in (W.WS_F_OBS, W.WS_F_ACTION, W.WS_F_LOGP, W.WS_F_POLICY_OUT)])
+            r.close()
+        assert np.isinf(rows[0][0]).any() and np.isfinite(rows[0][3]).all()
+        for x, y in zip(*rows):
+            assert np.array_equal(x.view(np.uint8), y.view(np.uint8)), n

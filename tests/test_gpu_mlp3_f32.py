@@ -71,3 +71,27 @@ def test_noalloc_forward_edges(rows, widths):
     (2431, (4, 64, 64, 16)), (8, (24, 33, 64, 48))])
 def test_noalloc_forward_few_rows(rows, widths):
     test_noalloc_forward_edges(rows, widths)
+
+
+@pytest.mark.parametrize("rows,widths", [
+    (9, (3, 33, 37, 5)), (300, (4, 61, 100, 20)), (9, (30, 33, 37, 60)), (9, (5, 250, 130, 3)),
+    (4900, (4, 66, 66, 2)), (31000, (4, 61, 33, 2)), (9000, (7, 129, 250, 4))])
+def test_infinite_inputs_match_the_layers(rows, widths):
+    # a unit past the width sees inf * 0: it must stay out of the next layer, as in the layer-by-layer forward
+    torch = need_gpu()
+    g = inputs.rng(rows)
+    p = torch.from_numpy(inputs.policy_params(g, list(widths), scale=2.0)).cuda()
+    x = g.uniform(-1, 1, (rows, widths[0])).astype(np.float32)
+    x[1, 0], x[rows - 1, widths[0] - 1] = np.inf, -np.inf
+    x[rows // 2, 1] = np.nan
+    got = []
+    for over in (False, True):
+        buf = torch.zeros(rows * max(widths[0], widths[3]), device="cuda")
+        obs = buf[:rows * widths[0]]
+        obs.copy_(torch.from_numpy(x).reshape(-1))
+        out = buf if over else torch.empty(rows * widths[3], device="cuda")
+        assert W.ws_policy_forward_noalloc(obs.data_ptr(), rows, p.data_ptr(), *widths, out.data_ptr(),
+                                           torch.cuda.current_stream().cuda_stream) == W.WS_OK
+        got.append(out[:rows * widths[3]].cpu().numpy().reshape(rows, widths[3]))
+    assert np.isnan(got[1]).sum() == widths[3]  # the row with a NaN input, no other
+    assert np.array_equal(got[0], got[1], equal_nan=True)
