@@ -1,5 +1,5 @@
-// ws_gemm_tc.cu -- FP32-accurate GEMMs of the actor-critic update on the
-// tensor cores (tcgen05).
+// ws_gemm_tc.cu -- FP32-accurate GEMMs of the actor-critic update on the tensor
+// cores (tcgen05), for the shapes that ws_train_fwd.cu and ws_train_bwd.cu do not hold.
 //
 // Paper grounding: Sec. 2 and App. B keep training on the GPU, fed in place by
 // the roll-out store; the update's three hidden-by-hidden products per network

@@ -4,7 +4,8 @@
 //
 // Every kernel here is one launch per sub-step per step: this is the
 // one-launch-per-step FP32 baseline (and, captured in a CUDA graph, the
-// batched-FP32 path).  The fused tensor-core path lives in ws_control_tc.cu.
+// batched-FP32 path where ws_control_f32.cu and ws_mlp3_f32.cu do not take over).  The
+// fused tensor-core path lives in ws_control_tc.cu.
 #include <math.h>
 
 #include "ws_acrobot.cuh"

@@ -9,7 +9,9 @@
 // tiles; layer 2 as three tcgen05 products per K step (as k_gemm_tc); tanhf, h2
 // written; the output layer in FP32 FMAs.  The parts ran as a gather, a thin GEMM,
 // a 128 x 128-tile GEMM that read h1 twice, and a thin output layer (65,536 rows x
-// 4-256-256-2: 20 + 63 + 17 us with a 64 MB activation read between each).
+// 4-256-256-2: 20 + 63 + 17 us per network with a 64 MB activation read between each);
+// here 58,368 rows of both networks take 87 us, bound by the issue slots and the SFU
+// (60 M tanhf of two SFU results each).
 #include <math.h>
 
 #include "ws_train_tc.cuh"
