@@ -910,11 +910,11 @@ ws_status ws_rollout(ws_ctx *c, uint32_t n) {
   if (c->cfg.path == WS_PATH_PLAIN_FP32) {
     for (uint32_t i = 0; i < n && s == WS_OK; ++i) s = enqueue_steps(c, 1, c->stream);
   } else if (fused(c) || fused_f32_control(c)) {
-    // one kernel per chunk: a few launches cost the host what a graph's does, without
-    // the capture that a new context, launch configuration or seed pays for the graph
-    // (kGraphChunks below: one chunk 5 us either way, the capture and upload 90 us)
-    constexpr uint32_t kGraphChunks = 4;
-    if ((n + chunk_of(c) - 1) / chunk_of(c) < kGraphChunks) {
+    // a single chunk: its launches cost the host what a graph's does (5 us either way),
+    // without the capture and upload (90 us) that a new context, launch configuration or
+    // seed pays; with more chunks the graph's shorter gaps count (119 us against 123
+    // launched one by one for a short roll-out)
+    if (n <= chunk_of(c)) {
       s = enqueue_steps(c, n, c->stream);
     } else {
       cudaGraphExec_t g;
