@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <utility>
+
 #include "../../include/warpsci.h"
 
 #define WS_HD __host__ __device__ __forceinline__
@@ -100,6 +102,29 @@ __device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) {
   uint64_t d;
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
   return d;
+}
+
+// Launch a kernel and return this launch's own status.  (cudaGetLastError() after
+// <<<>>> also returns, and clears, an error that an earlier call of the thread left.)
+template <typename... P, typename... A>
+inline cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
+                                 cudaStream_t st, A &&...args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
+
+// A kernel's limit of dynamic shared memory.  (A successful cudaFuncSetAttribute clears the
+// thread's last error, and with it that of a refused launch before: while there is one,
+// it is returned instead, and stays for the caller's check.)
+template <typename K>
+inline cudaError_t set_smem_limit(K *kernel, int bytes) {
+  const cudaError_t pending = cudaPeekAtLastError();
+  if (pending != cudaSuccess) return pending;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
 }
 
 WS_HD uint32_t bounded(uint32_t w, uint32_t n) { return mul_hi32(w, n); }

@@ -298,17 +298,15 @@ cudaError_t run_gemm(dim3 g, cudaStream_t st, const float *A, int lda, const flo
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev < 0 || dev >= 64 || !attr_set[dev]) {
-    const cudaError_t e = cudaFuncSetAttribute(k_gemm_tc<TA, TB, EPI>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+    const cudaError_t e = set_smem_limit(k_gemm_tc<TA, TB, EPI>, kSmem);
     if (e != cudaSuccess) return e;
     if (dev >= 0 && dev < 64) attr_set[dev] = true;
   }
   // 16-byte loads along k where rows start on 16-byte boundaries
   const bool va = !TA && lda % 4 == 0 && ((uintptr_t)A & 15) == 0;
   const bool vb = TB && ldb % 4 == 0 && ((uintptr_t)B & 15) == 0;
-  k_gemm_tc<TA, TB, EPI><<<g, kThreads, kSmem, st>>>(A, lda, B, ldb, C, M, N, k_lo, k_hi, k_slice,
-                                                     slice_stride, aux, va, vb, err);
-  return cudaGetLastError();
+  return launch_kernel(k_gemm_tc<TA, TB, EPI>, g, dim3(kThreads), kSmem, st, A, lda, B, ldb, C, M, N, k_lo, k_hi,
+                       k_slice, slice_stride, aux, va, vb, err);
 }
 
 }  // namespace

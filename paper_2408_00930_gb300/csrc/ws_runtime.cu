@@ -71,6 +71,10 @@ ws_status cuda_check(ws_ctx *c, cudaError_t e, const char *where) {
   return fail(c, WS_ERR_CUDA, std::string(where) + ": " + cudaGetErrorString(e));
 }
 
+// An error that an earlier call of this thread left in the runtime was that call's to
+// report: it is not taken for a failure of the launches that follow.
+void drop_earlier_error() { cudaGetLastError(); }
+
 ws_status validate(const ws_config *cfg) {
   if (!cfg || cfg->struct_size != sizeof(ws_config)) return WS_ERR_INVALID;
   if (cfg->env < WS_ENV_CONTROL || cfg->env > WS_ENV_ACROBOT) return WS_ERR_INVALID;
@@ -957,6 +961,7 @@ ws_status ws_a2c_update(ws_ctx *c, uint32_t n, float lr, float c_v, float c_e, d
   const TrainBufs tb = train_bufs((uint8_t *)c->state + c->L.train_off, c->L.pol);
   TrainGroup g[2];
   const int ng = train_groups(c, g);
+  drop_earlier_error();
   launch_returns(c->d, n, c->stream);
   launch_a2c_update(c->d, tb, g, ng, n, lr, c_v, c_e, c->stream);
   return finish_update(c, tb, n, stats, 3, "a2c update");
@@ -970,6 +975,7 @@ ws_status ws_advantages(ws_ctx *c, uint32_t n) {
   const TrainBufs tb = train_bufs((uint8_t *)c->state + c->L.train_off, c->L.pol);
   TrainGroup g[2];
   const int ng = train_groups(c, g);
+  drop_earlier_error();
   launch_returns(c->d, n, c->stream);
   launch_advantages(c->d, tb, g, ng, n, c->stream);
   ws_status s = cuda_check(c, cudaGetLastError(), "advantages");
@@ -993,6 +999,7 @@ ws_status ws_ppo_update(ws_ctx *c, uint32_t n, float lr, float eps, float c_v, f
   const TrainBufs tb = train_bufs((uint8_t *)c->state + c->L.train_off, c->L.pol);
   TrainGroup g[2];
   const int ng = train_groups(c, g);
+  drop_earlier_error();
   launch_ppo_update(c->d, tb, g, ng, n, lr, eps, c_v, c_e, c->stream);
   return finish_update(c, tb, n, stats, 4, "ppo update");
 }

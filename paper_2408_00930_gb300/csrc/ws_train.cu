@@ -735,6 +735,17 @@ inline dim3 ggrid(int M, int N, int z = 1) {
   return dim3((unsigned)((M + kGM - 1) / kGM), (unsigned)((N + kGN - 1) / kGN), (unsigned)z);
 }
 
+// A launch that has a substitute: true if it was accepted.  A refused one's error is
+// cleared, so that the substitute decides the update's status; an error that was
+// there before it stays for the update's own check.
+template <typename F>
+bool accepted(F launch) {
+  const cudaError_t before = cudaPeekAtLastError();
+  if (launch() == cudaSuccess) return true;
+  if (before == cudaSuccess) cudaGetLastError();
+  return false;
+}
+
 // A hidden-layer GEMM of the update: on tcgen05 with FP32 operands split into
 // BF16 hi + lo (ws_gemm_tc.cu), or on the FP32 CUDA cores when the launch asks
 // for them (ws_launch.update_gemm).  The epilogue codes are shared.
@@ -747,8 +758,10 @@ void hgemm(const Dev &d, dim3 g, cudaStream_t st, const float *A, int lda, const
            const float *aux) {
   // a tensor-core launch that is refused (a shape it does not take) falls back
   // to the CUDA-core GEMM
-  if (!d.update_simt && launch_gemm_tc(TA, TB, EPI, A, lda, B, ldb, C, M, N, k_lo, k_hi, k_slice,
-                                       slice_stride, aux, d.err, st) == cudaSuccess)
+  if (!d.update_simt && accepted([&] {
+        return launch_gemm_tc(TA, TB, EPI, A, lda, B, ldb, C, M, N, k_lo, k_hi, k_slice, slice_stride,
+                              aux, d.err, st);
+      }))
     return;
   sgemm<TA, TB, EPI>(g, st, A, lda, B, ldb, C, M, N, k_lo, k_hi, k_slice, slice_stride, aux);
 }
@@ -797,19 +810,28 @@ void mlp_forward(const Dev &d, const PolicyShape &sh, const float *params, const
 // The fused kernels' shapes, unless the launch asks for FP32 CUDA-core GEMMs.
 bool use_train_tc(const Dev &d, const PolicyShape &p) { return !d.update_simt && train_tc_supported(p); }
 
+// The layer-by-layer path's inputs of a chunk, into tb.x.
+void gather(const Dev &d, const TrainBufs &tb, const TrainGroup &G, uint32_t n, size_t q0, int rows,
+            cudaStream_t st) {
+  k_a2c_gather<<<nblk(rows, 256), 256, 0, st>>>(d, n, q0, (uint32_t)rows, G.slot0, G.n_slots, G.pol.w[0],
+                                                tb);
+}
+
 // Forward of a chunk (rows from q0 of the group) through the policy (unless
-// critic_only) and the critic: one fused launch where the shape allows it, else
-// layer by layer from the gathered inputs.
-void chunk_forward(const Dev &d, const TrainBufs &tb, const TrainGroup &G, uint32_t n, size_t q0,
+// critic_only) and the critic: one fused launch where the shape allows it (true), else,
+// or if that launch is refused, layer by layer from the gathered inputs (false).
+bool chunk_forward(const Dev &d, const TrainBufs &tb, const TrainGroup &G, uint32_t n, size_t q0,
                    int rows, bool critic_only, cudaStream_t st) {
   if (use_train_tc(d, G.pol) &&
-      launch_train_fwd(d, G, tb, q0, n, (uint32_t)rows, critic_only, st) == cudaSuccess) {
+      accepted([&] { return launch_train_fwd(d, G, tb, q0, n, (uint32_t)rows, critic_only, st); })) {
     if (!critic_only && !train_fwd_has_out(G.pol.w[3]))
       mlp_forward(d, G.pol, G.params, tb.x, tb.h1, tb.h2, tb.out, rows, st, 2);
-    return;
+    return true;
   }
+  gather(d, tb, G, n, q0, rows, st);
   if (!critic_only) mlp_forward(d, G.pol, G.params, tb.x, tb.h1, tb.h2, tb.out, rows, st);
   mlp_forward(d, G.crit, G.critic, tb.x, tb.c1, tb.c2, tb.vout, rows, st);
+  return false;
 }
 
 // Rows per chunk: whole rounds of 128-row tiles over the SMs for the fused
@@ -826,13 +848,14 @@ size_t chunk_rows(const Dev &d, const PolicyShape &p) {
 // Backward through one three-layer MLP for a chunk: X [rows][w0], h1, h2 the
 // tanh activations, dout [rows][w3] the gradient at the output.  Per layer the
 // weight gradient as row-slice partials (and the bias row), summed into
-// grad in slice order, then the data gradient into the layer below.
+// grad in slice order, then the data gradient into the layer below (d2: layer 2's,
+// d1: layer 1's).  Layers first to last; from layer 1 on, d2 is given.
 void mlp_backward(const Dev &d, const PolicyShape &sh, const float *params, const float *X,
                   const float *h1, const float *h2, const float *dout, float *grad, float *d1, float *d2,
-                  float *part, int rows, cudaStream_t st, int last = 0) {
+                  float *part, int rows, cudaStream_t st, int first = 2, int last = 0) {
   const float *ain[3] = {X, h1, h2};
   float *dl[3] = {nullptr, d1, d2};
-  for (int l = 2; l >= last; --l) {
+  for (int l = first; l >= last; --l) {
     const int M = sh.w[l], N = sh.w[l + 1];
     const int sr = slice_rows(M, N), nz = (rows + sr - 1) / sr;
     const float *D = l == 2 ? dout : dl[l + 1];
@@ -869,16 +892,27 @@ void mlp_backward(const Dev &d, const PolicyShape &sh, const float *params, cons
   }
 }
 
-// Backward of a chunk through both networks, the gradients added to tb.grad.
+// Backward of a chunk through both networks, the gradients added to tb.grad.  fused: as
+// chunk_forward ran (the fused kernel reads whole tiles of activations, which only the
+// fused forward fills).  A refused fused launch has added nothing to tb.grad (its last
+// kernel does), so the layers take its place from where the launch would have begun.
 void chunk_backward(const Dev &d, const TrainBufs &tb, const TrainGroup &G, uint32_t n, size_t q0,
-                    int rows, cudaStream_t st) {
+                    int rows, bool fused, cudaStream_t st) {
   float *ga = tb.grad, *gc = tb.grad + G.pol.count();
-  if (use_train_tc(d, G.pol)) {
-    if (!train_bwd_has_out(G.pol)) {  // the output layers, down to the gradients d1 (actor), d2 (critic)
-      mlp_backward(d, G.pol, G.params, tb.x, tb.h1, tb.h2, tb.out, ga, nullptr, tb.d1, tb.part, rows, st, 2);
-      mlp_backward(d, G.crit, G.critic, tb.x, tb.c1, tb.c2, tb.vout, gc, nullptr, tb.d2, tb.part, rows, st, 2);
+  if (fused) {
+    const bool has = train_bwd_has_out(G.pol);
+    if (!has) {  // the output layers, down to the gradients d1 (actor), d2 (critic)
+      mlp_backward(d, G.pol, G.params, tb.x, tb.h1, tb.h2, tb.out, ga, nullptr, tb.d1, tb.part, rows, st, 2, 2);
+      mlp_backward(d, G.crit, G.critic, tb.x, tb.c1, tb.c2, tb.vout, gc, nullptr, tb.d2, tb.part, rows, st, 2,
+                   2);
     }
-    if (launch_train_bwd(d, G, tb, q0, n, (uint32_t)rows, st) == cudaSuccess) return;
+    if (accepted([&] { return launch_train_bwd(d, G, tb, q0, n, (uint32_t)rows, st); })) return;
+    gather(d, tb, G, n, q0, rows, st);
+    if (!has) {  // (h2, read for the last time by the output layers, takes the next gradient)
+      mlp_backward(d, G.pol, G.params, tb.x, tb.h1, nullptr, nullptr, ga, tb.h2, tb.d1, tb.part, rows, st, 1);
+      mlp_backward(d, G.crit, G.critic, tb.x, tb.c1, nullptr, nullptr, gc, tb.c2, tb.d2, tb.part, rows, st, 1);
+      return;
+    }
   }
   mlp_backward(d, G.pol, G.params, tb.x, tb.h1, tb.h2, tb.out, ga, tb.d1, tb.d2, tb.part, rows, st);
   mlp_backward(d, G.crit, G.critic, tb.x, tb.c1, tb.c2, tb.vout, gc, tb.d1, tb.d2, tb.part, rows, st);
@@ -955,18 +989,16 @@ void run_update(const Dev &d, const TrainBufs &tb, const TrainGroup *groups, int
     if (use_train_tc(d, G.pol)) launch_train_pack(G, tb.image, st);
     for (size_t q0 = 0; q0 < R; q0 += CH) {
       const int rows = (int)((R - q0) < CH ? (R - q0) : CH);
-      if (!use_train_tc(d, G.pol))
-        k_a2c_gather<<<nblk(rows, 256), 256, 0, st>>>(d, n, q0, (uint32_t)rows, G.slot0, G.n_slots,
-                                                      G.pol.w[0], tb);
-      chunk_forward(d, tb, G, n, q0, rows, false, st);
+      const bool fused = chunk_forward(d, tb, G, n, q0, rows, false, st);
       if (ppo)
         k_ppo_head<<<nblk(rows, 256), 256, 0, st>>>(d, n, q0, (uint32_t)rows, G.slot0, G.n_slots,
                                                     G.pol.w[3], inv_r, eps, c_v, c_e, tb);
       else
         k_a2c_head<<<nblk(rows, 256), 256, 0, st>>>(d, n, q0, (uint32_t)rows, G.slot0, G.n_slots,
                                                     G.pol.w[3], inv_r, c_v, c_e, tb);
-      chunk_backward(d, tb, G, n, q0, rows, st);
+      chunk_backward(d, tb, G, n, q0, rows, fused, st);
     }
+    if (cudaPeekAtLastError() != cudaSuccess) return;  // a launch was lost: no step on such a gradient
     k_sgd<<<nblk(na, 256), 256, 0, st>>>(G.params, ga, na, lr);
     k_sgd<<<nblk(nc, 256), 256, 0, st>>>(G.critic, gc, nc, lr);
   }
@@ -995,9 +1027,6 @@ void launch_advantages(const Dev &d, const TrainBufs &tb, const TrainGroup *grou
     if (use_train_tc(d, G.pol)) launch_train_pack(G, tb.image, st);
     for (size_t q0 = 0; q0 < R; q0 += CH) {
       const int rows = (int)((R - q0) < CH ? (R - q0) : CH);
-      if (!use_train_tc(d, G.pol))
-        k_a2c_gather<<<nblk(rows, 256), 256, 0, st>>>(d, n, q0, (uint32_t)rows, G.slot0, G.n_slots,
-                                                      G.pol.w[0], tb);
       chunk_forward(d, tb, G, n, q0, rows, !both, st);
       k_adv_store<<<nblk(rows, 256), 256, 0, st>>>(d, n, q0, (uint32_t)rows, G.slot0, G.n_slots,
                                                    tb);

@@ -662,11 +662,9 @@ int sm_count() {
 template <int H, int XP, int OUT>
 cudaError_t run_bwd(const Dev &d, const Rows &rw, int in, const BNets &nets, int grid, cudaStream_t st) {
   using S = BwdSmem<H, XP, OUT>;
-  cudaError_t e = cudaFuncSetAttribute(k_train_bwd<H, XP, OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       S::BYTES);
+  cudaError_t e = set_smem_limit(k_train_bwd<H, XP, OUT>, S::BYTES);
   if (e != cudaSuccess) return e;
-  k_train_bwd<H, XP, OUT><<<grid, kThreads, S::BYTES, st>>>(d, rw, in, nets);
-  return cudaGetLastError();
+  return launch_kernel(k_train_bwd<H, XP, OUT>, dim3(grid), dim3(kThreads), S::BYTES, st, d, rw, in, nets);
 }
 
 // The output widths come with their input widths (control 4 -> 2, acrobot 6 -> 3,
@@ -689,10 +687,10 @@ template <int H>
 cudaError_t run_wgrad(const WNet &a, const WNet &c, int rows, int slices, int per, uint32_t *err,
                       cudaStream_t st) {
   using G = WGeo<H>;
-  cudaError_t e = cudaFuncSetAttribute(k_train_wgrad<H>, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM);
+  cudaError_t e = set_smem_limit(k_train_wgrad<H>, G::SMEM);
   if (e != cudaSuccess) return e;
-  k_train_wgrad<H><<<dim3((unsigned)slices, G::MH, 2), kWT, G::SMEM, st>>>(a, c, rows, per, err);
-  return cudaGetLastError();
+  return launch_kernel(k_train_wgrad<H>, dim3((unsigned)slices, G::MH, 2), dim3(kWT), G::SMEM, st, a, c, rows,
+                       per, err);
 }
 
 }  // namespace
@@ -765,8 +763,7 @@ cudaError_t launch_train_bwd(const Dev &d, const TrainGroup &g, const TrainBufs 
     seg(p3a, ga + g.pol.layer_offset(2), grid, l3a);
     seg(p3c, gc + g.crit.layer_offset(2), grid, l3c);
   }
-  k_train_reduce<<<blocks, 512, 0, st>>>(s);
-  return cudaGetLastError();
+  return launch_kernel(k_train_reduce, dim3(blocks), dim3(512), 0, st, s);
 }
 
 }  // namespace ws

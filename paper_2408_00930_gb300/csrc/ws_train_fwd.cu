@@ -293,11 +293,11 @@ template <int H, int OUT, int XV>
 cudaError_t run_fwd_x(const Dev &d, const Rows &rw, int in, const Nets &nets, cudaStream_t st) {
   const int xp = (in + 3) & ~3, out = OUT > 1 ? OUT : 1, smem = FwdSmem<H>::bytes(in, xp, out);
   const int off_w = FwdSmem<H>::w_fits(in, xp, out) ? FwdSmem<H>::off_w(xp) : 0;
-  cudaError_t e = cudaFuncSetAttribute(k_train_fwd<H, OUT, XV>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaError_t e = set_smem_limit(k_train_fwd<H, OUT, XV>, smem);
   if (e != cudaSuccess) return e;
   const int tiles = nets.count * (int)((rw.rows + kRows - 1) / kRows), ctas = 2 * sm_count();
-  k_train_fwd<H, OUT, XV><<<tiles < ctas ? tiles : ctas, kThreads, smem, st>>>(d, rw, in, xp, off_w, nets);
-  return cudaGetLastError();
+  return launch_kernel(k_train_fwd<H, OUT, XV>, dim3(tiles < ctas ? tiles : ctas), dim3(kThreads), smem, st, d,
+                       rw, in, xp, off_w, nets);
 }
 template <int H, int OUT>
 cudaError_t run_fwd(const Dev &d, const Rows &rw, int in, const Nets &nets, cudaStream_t st) {

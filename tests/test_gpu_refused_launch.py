@@ -1,0 +1,126 @@
+"""Launches that the runtime refuses: each launch of a call in turn, in a process of its own with tests/refuse_launch.cpp
+ahead of the library.  A call that lost a launch reports it, unless something took the launch's place: then what it
+gives is right.
+
+Updates: the parameter change is the undisturbed update's within the two paths' error (2e-4 of the largest gradient
+and the half ulp of a parameter, as the fused update against the FP32 one), with the output layers in the fused
+kernels and outside, over one chunk and two with a partial last tile."""
+import ctypes
+import os
+import subprocess
+import sys
+
+import numpy as np
+import pytest
+
+from paper_2408_00930_gb300 import build
+from paper_2408_00930_gb300 import warpsci as W
+from tests.gpu_common import need_gpu
+
+pytestmark = pytest.mark.gpu
+HERE = os.path.dirname(os.path.abspath(__file__))
+LR = 1.0
+
+# algorithm, env, hidden width, envs, steps, dimension
+UPDATES = [("a2c", W.WS_ENV_CONTROL, 128, 5000, 14, 0), ("ppo", W.WS_ENV_CONTROL, 64, 129, 2, 0),
+           ("ppo", W.WS_ENV_LANDSCAPE, 128, 5000, 14, 9), ("a2c", W.WS_ENV_LANDSCAPE, 64, 130, 2, 5),
+           ("ppo", W.WS_ENV_ECONOMY, 256, 5, 3, 0)]
+
+
+def context(env, h, n, T, dim, flags=0, path=W.WS_PATH_BATCHED_FP32):
+    kw = {}
+    if env == W.WS_ENV_LANDSCAPE:
+        kw.update(dim=dim, n_gauss=64)
+    if env == W.WS_ENV_ECONOMY:
+        kw["agents_per_env"] = np.random.default_rng(2).integers(100, 200, n)
+    r = W.Rollout(env, path, n, T, 9, h, h, param_seed=5, flags=flags, **kw)
+    r.reset(6)
+    return r
+
+
+def update(algo, env, h, n, T, dim, arm=lambda: None, disarm=lambda: None):
+    """(status, before, after, advantages) of one update; arm() before its calls, disarm() after."""
+    r = context(env, h, n, T, dim, W.WS_FLAG_TRAIN | W.WS_FLAG_BOUNDS_CHECK)
+    r.rollout(T)
+    nets = [(r.obs_dim(), r.n_out())] + ([(16, 10)] if env == W.WS_ENV_ECONOMY else [])
+    count = lambda a, b: a * h + h + h * h + h + h * b + b  # noqa: E731
+    sizes = {W.WS_F_PARAMS: sum(count(*s) for s in nets), W.WS_F_CRITIC: sum(count(s[0], 1) for s in nets)}
+    get = lambda: [r.fetch_raw(f, 4 * s).view(np.float32).copy() for f, s in sizes.items()]  # noqa: E731
+    before, adv = get(), None
+    arm()
+    if algo == "a2c":
+        st = W.ws_a2c_update(r.ctx, T, LR, 0.5, 0.01)
+    else:
+        st = W.ws_advantages(r.ctx, T)
+        if st == W.WS_OK:
+            st = W.ws_ppo_update(r.ctx, T, LR, 0.2, 0.5, 0.01)
+    disarm()
+    if st != W.WS_OK:
+        assert W.ws_last_error(r.ctx)
+        r.close()
+        return st, before, None, None
+    r.sync()
+    after = get()
+    if algo == "ppo":
+        adv = r.fetch(W.WS_F_ADVANTAGE, 0, T)
+    r.close()
+    return st, before, after, adv
+
+
+def check(ref, got):
+    for b, a, b2, a2 in zip(ref[1], ref[2], got[1], got[2]):
+        assert np.array_equal(b, b2)
+        g, g2 = b.astype(np.float64) - a, b.astype(np.float64) - a2
+        tol = 2e-4 * np.abs(g).max() + 1.2 * np.spacing(np.maximum(np.abs(a), np.abs(b)))
+        assert np.abs(g).max() > 0
+        assert np.all(np.abs(g - g2) <= tol), (np.abs(g - g2).max(), np.abs(g).max())
+    if ref[3] is not None:
+        assert np.abs(ref[3] - got[3]).max() <= 1e-4 * max(1.0, np.abs(ref[3]).max())
+
+
+# ---- in the process with the launch entries replaced: `rt` is that library
+def refuse_updates(rt, case):
+    ref = update(*case, arm=lambda: rt.refuse_launch(-1))
+    assert ref[0] == W.WS_OK
+    n, lost = rt.launches_seen(), 0
+    assert n >= 8
+    for i in range(n):
+        got = update(*case, arm=lambda: rt.refuse_launch(i), disarm=lambda: rt.refuse_launch(-1))
+        if got[0] == W.WS_OK:
+            check(ref, got)
+        else:
+            assert got[0] == W.WS_ERR_CUDA
+            lost += 1
+    assert 0 < lost < n  # plain launches have no substitute, the fused ones have
+
+
+def child(what, tmp_path, *args):
+    lib = str(tmp_path / "refuse.so")
+    inc = os.path.join(os.path.dirname(build.nvcc()), "..", "include")
+    subprocess.run(["g++", "-shared", "-fPIC", "-I", inc, os.path.join(HERE, "refuse_launch.cpp"), "-o", lib, "-ldl"],
+                   check=True)
+    code = ("import ctypes, sys; rt = ctypes.CDLL(sys.argv[1], mode=ctypes.RTLD_GLOBAL)\n"
+            "sys.path.insert(0, sys.argv[2])\n"
+            "from tests import test_gpu_refused_launch as t; t.need_gpu(); getattr(t, sys.argv[3])(rt, *eval(sys.argv[4]))\n")
+    subprocess.run([sys.executable, "-c", code, lib, os.path.dirname(HERE), what, repr(args)], check=True, timeout=600)
+
+
+@pytest.mark.parametrize("case", UPDATES)
+def test_updates(case, tmp_path):
+    need_gpu()
+    child("refuse_updates", tmp_path, case)
+
+
+@pytest.mark.parametrize("case", UPDATES)
+def test_earlier_error_is_not_the_updates(case):
+    # an error that another call of the thread left in the runtime
+    need_gpu()
+    rt = ctypes.CDLL("libcudart.so.13")
+
+    def leave_error():
+        assert rt.cudaSetDevice(1 << 20) != 0 and rt.cudaPeekAtLastError() != 0
+    ref = update(*case)
+    got = update(*case, arm=leave_error, disarm=rt.cudaGetLastError)
+    assert ref[0] == got[0] == W.WS_OK
+    for x, y in zip(ref[1] + ref[2], got[1] + got[2]):
+        assert np.array_equal(x, y)
