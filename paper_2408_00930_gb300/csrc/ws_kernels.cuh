@@ -88,7 +88,8 @@ struct Branch {
   cudaStream_t aux;
   cudaEvent_t fork, join;
 };
-void launch_plain_step(const Dev &d, uint32_t step_off, cudaStream_t st, const Branch *br);
+// (the status of a step's policy launches)
+cudaError_t launch_plain_step(const Dev &d, uint32_t step_off, cudaStream_t st, const Branch *br);
 void launch_advance(const Dev &d, uint32_t n, cudaStream_t st);
 
 // ---- S7: discounted returns ----------------------------------------------

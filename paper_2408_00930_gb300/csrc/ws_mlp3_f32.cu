@@ -200,10 +200,9 @@ cudaError_t run_u(const float *X, long ldr, long ldc, const float *params, const
                   float *Y, int M, cudaStream_t st) {
   const float *W0 = params + sh.layer_offset(0), *W1 = params + sh.layer_offset(1),
               *W2 = params + sh.layer_offset(2);
-  k_mlp3_f32u<HP><<<(unsigned)((M + 7) / 8), 128, 0, st>>>(
-      X, ldr, ldc, W0, W0 + (size_t)sh.w[0] * sh.w[1], W1, W1 + (size_t)sh.w[1] * sh.w[2], W2,
-      W2 + (size_t)sh.w[2] * sh.w[3], Y, M, sh.w[0], sh.w[1], sh.w[2], sh.w[3]);
-  return cudaGetLastError();
+  return launch_kernel(k_mlp3_f32u<HP>, dim3((unsigned)((M + 7) / 8)), dim3(128), 0, st, X, ldr, ldc, W0,
+                       W0 + (size_t)sh.w[0] * sh.w[1], W1, W1 + (size_t)sh.w[1] * sh.w[2], W2,
+                       W2 + (size_t)sh.w[2] * sh.w[3], Y, M, sh.w[0], sh.w[1], sh.w[2], sh.w[3]);
 }
 
 template <int NT, int TM, int CPT, int ST>
@@ -216,18 +215,16 @@ cudaError_t run(const float *X, long ldr, long ldc, const float *params, const P
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev < 0 || dev >= 64 || !attr_set[dev]) {
-    const cudaError_t e = cudaFuncSetAttribute(k_mlp3_f32<NT, TM, CPT, ST>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               C::floats(kMaxIn) * 4);
+    const cudaError_t e = set_smem_limit(k_mlp3_f32<NT, TM, CPT, ST>, C::floats(kMaxIn) * 4);
     if (e != cudaSuccess) return e;
     if (dev >= 0 && dev < 64) attr_set[dev] = true;
   }
   const float *W0 = params + sh.layer_offset(0), *W1 = params + sh.layer_offset(1),
               *W2 = params + sh.layer_offset(2);
-  k_mlp3_f32<NT, TM, CPT, ST><<<(unsigned)((M + C::RM - 1) / C::RM), NT, smem, st>>>(
-      X, ldr, ldc, W0, W0 + (size_t)sh.w[0] * sh.w[1], W1, W1 + (size_t)sh.w[1] * sh.w[2], W2,
-      W2 + (size_t)sh.w[2] * sh.w[3], Y, M, sh.w[0], sh.w[1], sh.w[2], sh.w[3]);
-  return cudaGetLastError();
+  return launch_kernel(k_mlp3_f32<NT, TM, CPT, ST>, dim3((unsigned)((M + C::RM - 1) / C::RM)), dim3(NT), smem,
+                       st, X, ldr, ldc, W0, W0 + (size_t)sh.w[0] * sh.w[1], W1,
+                       W1 + (size_t)sh.w[1] * sh.w[2], W2, W2 + (size_t)sh.w[2] * sh.w[3], Y, M, sh.w[0],
+                       sh.w[1], sh.w[2], sh.w[3]);
 }
 
 }  // namespace

@@ -62,10 +62,10 @@ extern "C" ws_status ws_policy_forward_noalloc(const float *obs, uint32_t n_rows
   const auto apart = [&](const float *p, size_t n) {
     return out + (size_t)n_rows * out_dim <= p || p + n <= out;
   };
-  if (ws::mlp3_f32_supported(sh) && apart(obs, (size_t)n_rows * in_dim) && apart(params, sh.count()))
-    return ws::launch_mlp3_f32(obs, in_dim, 1, params, sh, out, (int)n_rows, st) == cudaSuccess
-               ? WS_OK
-               : WS_ERR_CUDA;
+  if (ws::mlp3_f32_supported(sh) && apart(obs, (size_t)n_rows * in_dim) && apart(params, sh.count())) {
+    const cudaError_t e = ws::launch_mlp3_f32(obs, in_dim, 1, params, sh, out, (int)n_rows, st);
+    return cudaGetLastError() == cudaSuccess && e == cudaSuccess ? WS_OK : WS_ERR_CUDA;
+  }
   // Every element of h0 and h1 is written before it is read, so the contents
   // left by an earlier call need no clearing.
   ws::launch_dense_fp32(obs, in_dim, 1, W0, b0, h0, (int)n_rows, (int)in_dim, (int)hidden0, 1, st);

@@ -238,24 +238,28 @@ void mlp3(const float *X, long ldr, long ldc, const float *params, const PolicyS
 }
 
 // BF16 tensor-core variant: hidden activations in BF16 row-major, logits FP32.
-void tc_mlp3(const Dev &d, const float *X, long ldr, long ldc, const PolicyShape &sh, int pid,
+cudaError_t tc_mlp3(const Dev &d, const float *X, long ldr, long ldc, const PolicyShape &sh, int pid,
              void *h0, void *h1, float *out, long M, cudaStream_t st) {
-  launch_dense_tc(X, ldr, ldc, 0, sh.w[0], d.pk[pid][0], sh.w[1], h0, 1, 1, M, d.err, st);
-  launch_dense_tc(h0, 0, 0, 1, sh.w[1], d.pk[pid][1], sh.w[2], h1, 1, 1, M, d.err, st);
-  launch_dense_tc(h1, 0, 0, 1, sh.w[2], d.pk[pid][2], sh.w[3], out, 0, 0, M, d.err, st);
+  cudaError_t e = launch_dense_tc(X, ldr, ldc, 0, sh.w[0], d.pk[pid][0], sh.w[1], h0, 1, 1, M, d.err, st);
+  if (e == cudaSuccess) e = launch_dense_tc(h0, 0, 0, 1, sh.w[1], d.pk[pid][1], sh.w[2], h1, 1, 1, M, d.err, st);
+  if (e == cudaSuccess) e = launch_dense_tc(h1, 0, 0, 1, sh.w[2], d.pk[pid][2], sh.w[3], out, 0, 0, M, d.err, st);
+  return e;
 }
 
-void policy(const Dev &d, const float *X, long ldr, long ldc, const float *params,
+// A launcher's status is returned; that of the kernels launched in place is the
+// runtime's last error.
+cudaError_t policy(const Dev &d, const float *X, long ldr, long ldc, const float *params,
             const PolicyShape &sh, int pid, float *h0, float *h1, float *out, int M,
             cudaStream_t st) {
   if (d.mlp3)
     launch_mlp3_tc(X, ldr, ldc, d.pk[pid][0], sh, out, M, d.err, st);
   else if (d.fuse_mlp && mlp3_f32_supported(sh))
-    launch_mlp3_f32(X, ldr, ldc, params, sh, out, M, st);
+    return launch_mlp3_f32(X, ldr, ldc, params, sh, out, M, st);
   else if (d.tc_mlp)
-    tc_mlp3(d, X, ldr, ldc, sh, pid, h0, h1, out, M, st);
+    return tc_mlp3(d, X, ldr, ldc, sh, pid, h0, h1, out, M, st);
   else
     mlp3(X, ldr, ldc, params, sh, h0, h1, out, M, st);
+  return cudaSuccess;
 }
 
 // ------------------------------------------------- S1/S6 observation store
@@ -1038,16 +1042,17 @@ void launch_reset(const Dev &d, cudaStream_t st) {
   }
 }
 
-void launch_plain_step(const Dev &d, uint32_t off, cudaStream_t st, const Branch *br) {
+cudaError_t launch_plain_step(const Dev &d, uint32_t off, cudaStream_t st, const Branch *br) {
+  cudaError_t e = cudaSuccess;  // of the policies; the step's other launches follow all the same
   const int T = d.env_threads > 0 ? d.env_threads : 256;  // per-env kernels' block size
   if (d.env == WS_ENV_CONTROL) {
     k_store_obs<<<blocks(d.n_envs, T), T, 0, st>>>(d, off, d.s, 4, d.n_envs, d.n_envs, 0);
-    policy(d, d.s, 1, d.n_envs, d.params, d.pol, 0, d.h0, d.h1, d.out, (int)d.n_envs, st);
+    e = policy(d, d.s, 1, d.n_envs, d.params, d.pol, 0, d.h0, d.h1, d.out, (int)d.n_envs, st);
     k_sample_cat<<<blocks(d.n_envs, T), T, 0, st>>>(d, off, d.out, 2, 0, d.n_envs, 0);
     k_control_step<<<blocks(d.n_envs, T), T, 0, st>>>(d, off);
   } else if (d.env == WS_ENV_ACROBOT) {
     k_acrobot_observe<<<blocks(d.n_envs, T), T, 0, st>>>(d, off);
-    policy(d, d.pobs, 1, d.n_envs, d.params, d.pol, 0, d.h0, d.h1, d.out, (int)d.n_envs, st);
+    e = policy(d, d.pobs, 1, d.n_envs, d.params, d.pol, 0, d.h0, d.h1, d.out, (int)d.n_envs, st);
     k_sample_cat<<<blocks(d.n_envs, T), T, 0, st>>>(d, off, d.out, 3, 0, d.n_envs, 0);
     k_acrobot_step<<<blocks(d.n_envs, T), T, 0, st>>>(d, off);
   } else if (d.env == WS_ENV_ECONOMY) {
@@ -1059,12 +1064,13 @@ void launch_plain_step(const Dev &d, uint32_t off, cudaStream_t st, const Branch
       cudaStreamWaitEvent(br->aux, br->fork, 0);
       ps = br->aux;
     }
-    policy(d, d.pobs, kEconF, 1, d.params_planner, d.pol_planner, 1, d.ph0, d.ph1, d.pout,
-           (int)d.n_envs, ps);
+    e = policy(d, d.pobs, kEconF, 1, d.params_planner, d.pol_planner, 1, d.ph0, d.ph1, d.pout,
+               (int)d.n_envs, ps);
     k_sample_cat<<<blocks(d.n_envs, T), T, 0, ps>>>(d, off, d.pout, (int)d.n_out_planner, 2,
                                                          d.n_envs, d.n_agent_slots);
-    policy(d, d.feat, 1, d.n_agent_slots, d.params, d.pol, 0, d.h0, d.h1, d.out,
-           (int)d.n_agent_slots, st);
+    const cudaError_t ea = policy(d, d.feat, 1, d.n_agent_slots, d.params, d.pol, 0, d.h0, d.h1, d.out,
+                                  (int)d.n_agent_slots, st);
+    if (e == cudaSuccess) e = ea;
     k_sample_cat<<<blocks(d.n_agent_slots, T), T, 0, st>>>(d, off, d.out, (int)d.n_out, 1,
                                                                 d.n_agent_slots, 0);
     if (br) {
@@ -1075,13 +1081,14 @@ void launch_plain_step(const Dev &d, uint32_t off, cudaStream_t st, const Branch
     k_econ_finish<<<d.n_envs, kEconThreads, 0, st>>>(d, off);
   } else {
     k_store_obs<<<blocks(d.n_envs, T), T, 0, st>>>(d, off, d.s, (int)d.dim, d.n_envs, d.n_envs, 0);
-    policy(d, d.s, 1, d.n_envs, d.params, d.pol, 0, d.h0, d.h1, d.out, (int)d.n_envs, st);
+    e = policy(d, d.s, 1, d.n_envs, d.params, d.pol, 0, d.h0, d.h1, d.out, (int)d.n_envs, st);
     k_sample_gauss<<<blocks(d.n_envs, T), T, 0, st>>>(d, off);
     landscape_energy(d, off, 0, st);
     k_landscape_step<<<blocks(d.n_envs, T), T, 0, st>>>(d, off);
     landscape_energy(d, off, 1, st);
     k_landscape_reset_finish<<<blocks(d.n_envs, T), T, 0, st>>>(d, off, 0);
   }
+  return e;
 }
 
 void launch_advance(const Dev &d, uint32_t n, cudaStream_t st) { k_advance<<<1, 32, 0, st>>>(d, n); }

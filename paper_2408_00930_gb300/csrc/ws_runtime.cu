@@ -68,6 +68,7 @@ ws_status fail(ws_ctx *c, ws_status s, const std::string &m) {
 
 ws_status cuda_check(ws_ctx *c, cudaError_t e, const char *where) {
   if (e == cudaSuccess) return WS_OK;
+  cudaGetLastError();  // reported here: not left for another context's check
   return fail(c, WS_ERR_CUDA, std::string(where) + ": " + cudaGetErrorString(e));
 }
 
@@ -591,7 +592,10 @@ ws_status enqueue_steps(ws_ctx *c, uint32_t n, cudaStream_t st) {
     launch_advance(c->d, n, st);
   } else {
     const Branch *br = c->br.aux ? &c->br : nullptr;
-    for (uint32_t i = 0; i < n; ++i) launch_plain_step(c->d, i, st, br);
+    for (uint32_t i = 0; i < n; ++i) {
+      const cudaError_t e = launch_plain_step(c->d, i, st, br);
+      if (e != cudaSuccess) return cuda_check(c, e, "policy launch");
+    }
     launch_advance(c->d, n, st);
   }
   return cuda_check(c, cudaGetLastError(), "step launch");
@@ -609,6 +613,7 @@ ws_status graph_for(ws_ctx *c, uint32_t n, cudaGraphExec_t *out) {
   cudaGraph_t g = nullptr;
   e = cudaStreamEndCapture(c->capture, &g);
   if (s != WS_OK) {
+    cudaGetLastError();  // (a launch that is refused also ends the capture with an error)
     if (g) cudaGraphDestroy(g);
     return s;
   }
@@ -900,6 +905,7 @@ ws_status ws_reset(ws_ctx *c, uint64_t seed) {
 ws_status ws_step(ws_ctx *c) {
   if (!c) return WS_ERR_INVALID;
   if (c->err != WS_OK) return c->err;
+  drop_earlier_error();
   ws_status s = enqueue_steps(c, 1, c->stream);
   c->ring_gen += 1;
   if (s == WS_OK) c->k_host += 1;
@@ -910,6 +916,7 @@ ws_status ws_rollout(ws_ctx *c, uint32_t n) {
   if (!c) return WS_ERR_INVALID;
   if (c->err != WS_OK) return c->err;
   if (n == 0) return WS_OK;
+  drop_earlier_error();
   ws_status s = WS_OK;
   if (c->cfg.path == WS_PATH_PLAIN_FP32) {
     for (uint32_t i = 0; i < n && s == WS_OK; ++i) s = enqueue_steps(c, 1, c->stream);

@@ -124,3 +124,58 @@ def test_earlier_error_is_not_the_updates(case):
     assert ref[0] == got[0] == W.WS_OK
     for x, y in zip(ref[1] + ref[2], got[1] + got[2]):
         assert np.array_equal(x, y)
+
+
+def refuse_rollouts(rt):
+    """Every launch of a roll-out (captured) and of a step (direct), on the FP32 paths and the BF16 path's layers."""
+    for path in (W.WS_PATH_BATCHED_FP32, W.WS_PATH_PLAIN_FP32, W.WS_PATH_BATCHED_BF16):
+        for env, n in ((W.WS_ENV_ECONOMY, 5), (W.WS_ENV_LANDSCAPE, 20), (W.WS_ENV_CONTROL, 20)):
+            for call in (lambda r: W.ws_rollout(r.ctx, 2), lambda r: W.ws_step(r.ctx)):
+                def run(i):
+                    r = context(env, 64, n, 4, 8, path=path)
+                    rt.refuse_launch(i)
+                    st, seen = call(r), rt.launches_seen()
+                    rt.refuse_launch(-1)
+                    again = W.ws_step(r.ctx)
+                    r.close()
+                    return seen, st, again
+                seen, st, again = run(-1)
+                assert st == again == W.WS_OK
+                for i in range(seen):
+                    assert run(i)[1:] == (W.WS_ERR_CUDA, W.WS_ERR_CUDA), (path, env, i)
+
+
+def refuse_forward(rt):
+    import torch
+    x, w, y = (torch.zeros(4096, device="cuda") for _ in range(3))
+
+    def call(out):
+        return W.ws_policy_forward_noalloc(x.data_ptr(), 3, w.data_ptr(), 4, 16, 16, 2, out.data_ptr(), 0)
+    for out in (y, x):  # one launch; over the input, layer by layer
+        rt.refuse_launch(-1)
+        assert call(out) == W.WS_OK
+        for i in range(rt.launches_seen()):
+            rt.refuse_launch(i)
+            assert call(out) == W.WS_ERR_CUDA
+        rt.refuse_launch(-1)
+        assert call(out) == W.WS_OK
+
+
+@pytest.mark.parametrize("what", ["refuse_rollouts", "refuse_forward"])
+def test_calls_without_a_substitute(what, tmp_path):
+    need_gpu()
+    child(what, tmp_path)
+
+
+@pytest.mark.parametrize("path", [W.WS_PATH_PLAIN_FP32, W.WS_PATH_BATCHED_FP32, W.WS_PATH_BATCHED_BF16])
+def test_earlier_error_is_not_the_rollouts(path):
+    need_gpu()
+    rt = ctypes.CDLL("libcudart.so.13")
+    for env in (W.WS_ENV_ECONOMY, W.WS_ENV_LANDSCAPE, W.WS_ENV_CONTROL):
+        r = context(env, 64, 5, 4, 8, path=path)
+        for call in (lambda: W.ws_step(r.ctx), lambda: W.ws_rollout(r.ctx, 2)):
+            assert rt.cudaSetDevice(1 << 20) != 0 and rt.cudaPeekAtLastError() != 0
+            assert call() == W.WS_OK
+        r.sync()
+        r.close()
+    rt.cudaGetLastError()
