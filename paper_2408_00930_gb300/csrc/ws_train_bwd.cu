@@ -285,7 +285,7 @@ __global__ void __launch_bounds__(kThreads, 2)
       for (int i = tid; i < no * H; i += kCT) w3t[i] = __ldg(net.W3 + (i % H) * no + i / H);
       const int mine = my_tiles(tiles, q), t0 = first_tile(tiles, q);
       float xn[XV];
-      if (mine > 0) load_x(d, rw, t0, in, xn);
+      if (mine > 0) load_x<false>(d, rw, t0, in, xn);
       for (int t = 0; t < mine && ok; ++t) {
         const int tile = t0 + t * (int)gridDim.x;
         store_x(xn, XP, xs);
@@ -294,7 +294,7 @@ __global__ void __launch_bounds__(kThreads, 2)
           ds[i] = r < (int)rw.rows ? net.dout[(size_t)tile * kRows * no + i] : 0.f;
         }
         csync();
-        if (t + 1 < mine) load_x(d, rw, tile + (int)gridDim.x, in, xn);
+        if (t + 1 < mine) load_x<false>(d, rw, tile + (int)gridDim.x, in, xn);
         if (q == 0)
           ok = bwd_tile<H, XP, OUT, S::A1_SMEM>(net, bars, sm, xs, ds, w3t, a1, a3, in, (int)rw.rows,
                                                 tile, tmem, ph, ph_af);

@@ -160,7 +160,7 @@ __device__ __forceinline__ bool fwd_tile(const Net &net, Bars *bars, uint8_t *re
     if (lane == 0) arrive(&bars->a);
   }
   float xn[XV];
-  if (next >= 0) load_x(d, rw, next, in, xn);
+  if (next >= 0) load_x<true>(d, rw, next, in, xn);
   // ---- layer 2's accumulator, then tanh and the output layer
   const bool ok = call(tc::mbar_wait(&bars->acc, ph_acc, tc::kDrainNs) && okw);
   if (!ok) return false;
@@ -252,7 +252,7 @@ __global__ void __launch_bounds__(kThreads, 2)
       const int mine = my_tiles(tiles, q), out = q == 0 ? OUT : 1;
       if (mine == 0) continue;
       float xn[XV];
-      load_x(d, rw, first_tile(tiles, q), in, xn);
+      load_x<true>(d, rw, first_tile(tiles, q), in, xn);
       csync();  // the last network's weights and observations are read
       if (ws) {
         for (int i = tid; i < (in + 1) * H; i += kCT) ws[i] = __ldg(net.W1 + i);

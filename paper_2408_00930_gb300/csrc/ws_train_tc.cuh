@@ -248,15 +248,18 @@ __device__ __forceinline__ size_t ring_slot(const Dev &d, const Rows &rw, uint32
   return rw.slot0 + (size_t)s;
 }
 
-// The tile's observations for xs[row][xp], rows past the end zero: thread (row =
-// tid % 128, tid / 128) takes inputs tid / 128, + 2, ...; loaded into registers
-// while the tile before is still in work, then stored.
+// The tile's observations for xs[row][xp], rows past the end zero, or with REPEAT the last
+// row's (a zero input times an infinite weight is NaN, which would reach the sums over the
+// tile's rows through that row's zero gradients; the last row's activations are as finite
+// as the sums): thread (row = tid % 128, tid / 128) takes inputs tid / 128, + 2, ...;
+// loaded into registers while the tile before is still in work, then stored.
 constexpr int kXT = kCT / kRows;  // threads per row
 // (XV inputs per thread: as many as the network has over kXT)
-template <int XV>
+template <bool REPEAT, int XV>
 __device__ __forceinline__ void load_x(const Dev &d, const Rows &rw, int tile, int in, float (&v)[XV]) {
   const int tid = threadIdx.x, r = tid & 127;
-  const uint32_t i = (uint32_t)tile * kRows + (uint32_t)r;
+  uint32_t i = (uint32_t)tile * kRows + (uint32_t)r;
+  if (REPEAT) i = min(i, rw.rows - 1u);
   size_t row = 0, s = 0;
   const bool ok = i < rw.rows;
   if (ok) s = ring_slot(d, rw, i, &row);
