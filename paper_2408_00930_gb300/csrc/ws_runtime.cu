@@ -601,6 +601,15 @@ ws_status enqueue_steps(ws_ctx *c, uint32_t n, cudaStream_t st) {
   return cuda_check(c, cudaGetLastError(), "step launch");
 }
 
+// A caller's capture takes no roll-out: the steps would be counted (ws_get_step, ws_fetch)
+// without having run.  The graph launch of ws_rollout is refused by the runtime there.
+bool capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cs) == cudaSuccess) return cs != cudaStreamCaptureStatusNone;
+  drop_earlier_error();
+  return true;
+}
+
 ws_status graph_for(ws_ctx *c, uint32_t n, cudaGraphExec_t *out) {
   auto it = c->graphs.find(n);
   if (it != c->graphs.end()) {
@@ -925,7 +934,7 @@ ws_status ws_rollout(ws_ctx *c, uint32_t n) {
     // without the capture and upload (90 us) that a new context, launch configuration or
     // seed pays; with more chunks the graph's shorter gaps count (119 us against 123
     // launched one by one for a short roll-out)
-    if (n <= chunk_of(c)) {
+    if (n <= chunk_of(c) && !capturing(c->stream)) {
       s = enqueue_steps(c, n, c->stream);
     } else {
       cudaGraphExec_t g;

@@ -1,0 +1,41 @@
+"""Roll-outs of a single chunk, which are launched directly or through a graph: the same answers either way."""
+import ctypes
+
+import pytest
+
+from paper_2408_00930_gb300 import warpsci as W
+from tests.gpu_common import need_gpu
+
+pytestmark = pytest.mark.gpu
+
+# env, path, hidden width, extra configuration: the paths whose chunk is one launch
+SHAPES = [(W.WS_ENV_CONTROL, W.WS_PATH_BATCHED_BF16, 64, {}), (W.WS_ENV_ACROBOT, W.WS_PATH_BATCHED_BF16, 64, {}),
+          (W.WS_ENV_CONTROL, W.WS_PATH_BATCHED_FP32, 64, {}), (W.WS_ENV_ACROBOT, W.WS_PATH_BATCHED_FP32, 64, {}),
+          (W.WS_ENV_ECONOMY, W.WS_PATH_BATCHED_BF16, 128, {}),
+          (W.WS_ENV_LANDSCAPE, W.WS_PATH_BATCHED_BF16, 256, dict(dim=8, n_gauss=256))]
+
+
+@pytest.mark.parametrize("env,path,h,kw", SHAPES)
+def test_a_capturing_stream_takes_no_rollout(env, path, h, kw):
+    # its steps would be counted without having run; refused whether or not its graph is there already
+    torch = need_gpu()
+    rt = ctypes.CDLL("libcudart.so.13")
+    for warm in (0, 1, 20):
+        for mode in (0, 1, 2):
+            st = torch.cuda.Stream()
+            with torch.cuda.stream(st):
+                r = W.Rollout(env, path, 30, 40, 15, h, h, **kw)
+                r.reset(3)
+                for _ in range(warm):
+                    r.rollout(10)
+                torch.cuda.synchronize()
+                k, g = r.k, ctypes.c_void_p()
+                assert rt.cudaStreamBeginCapture(ctypes.c_void_p(st.cuda_stream), mode) == 0
+                got = W.ws_rollout(r.ctx, 10)
+                rt.cudaStreamEndCapture(ctypes.c_void_p(st.cuda_stream), ctypes.byref(g))
+                rt.cudaGetLastError()
+                if g.value:
+                    rt.cudaGraphDestroy(g)
+                assert got == W.WS_ERR_CUDA and r.k == k, (warm, mode)
+                r.close()
+    torch.cuda.synchronize()
