@@ -6,19 +6,15 @@ Updates: the parameter change is the undisturbed update's within the two paths' 
 and the half ulp of a parameter, as the fused update against the FP32 one), with the output layers in the fused
 kernels and outside, over one chunk and two with a partial last tile."""
 import ctypes
-import os
-import subprocess
-import sys
 
 import numpy as np
 import pytest
 
-from paper_2408_00930_gb300 import build
 from paper_2408_00930_gb300 import warpsci as W
 from tests.gpu_common import need_gpu
+from tests.refuse_launch import child
 
 pytestmark = pytest.mark.gpu
-HERE = os.path.dirname(os.path.abspath(__file__))
 LR = 1.0
 
 # algorithm, env, hidden width, envs, steps, dimension
@@ -94,21 +90,10 @@ def refuse_updates(rt, case):
     assert 0 < lost < n  # plain launches have no substitute, the fused ones have
 
 
-def child(what, tmp_path, *args):
-    lib = str(tmp_path / "refuse.so")
-    inc = os.path.join(os.path.dirname(build.nvcc()), "..", "include")
-    subprocess.run(["g++", "-shared", "-fPIC", "-I", inc, os.path.join(HERE, "refuse_launch.cpp"), "-o", lib, "-ldl"],
-                   check=True)
-    code = ("import ctypes, sys; rt = ctypes.CDLL(sys.argv[1], mode=ctypes.RTLD_GLOBAL)\n"
-            "sys.path.insert(0, sys.argv[2])\n"
-            "from tests import test_gpu_refused_launch as t; t.need_gpu(); getattr(t, sys.argv[3])(rt, *eval(sys.argv[4]))\n")
-    subprocess.run([sys.executable, "-c", code, lib, os.path.dirname(HERE), what, repr(args)], check=True, timeout=600)
-
-
 @pytest.mark.parametrize("case", UPDATES)
 def test_updates(case, tmp_path):
     need_gpu()
-    child("refuse_updates", tmp_path, case)
+    child("refuse_updates", tmp_path, case, module="test_gpu_refused_launch")
 
 
 @pytest.mark.parametrize("case", UPDATES)
@@ -164,7 +149,7 @@ def refuse_forward(rt):
 @pytest.mark.parametrize("what", ["refuse_rollouts", "refuse_forward"])
 def test_calls_without_a_substitute(what, tmp_path):
     need_gpu()
-    child(what, tmp_path)
+    child(what, tmp_path, module="test_gpu_refused_launch")
 
 
 @pytest.mark.parametrize("path", [W.WS_PATH_PLAIN_FP32, W.WS_PATH_BATCHED_FP32, W.WS_PATH_BATCHED_BF16])

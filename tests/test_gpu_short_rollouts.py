@@ -5,6 +5,7 @@ import pytest
 
 from paper_2408_00930_gb300 import warpsci as W
 from tests.gpu_common import need_gpu
+from tests.refuse_launch import child
 
 pytestmark = pytest.mark.gpu
 
@@ -39,3 +40,29 @@ def test_a_capturing_stream_takes_no_rollout(env, path, h, kw):
                 assert got == W.WS_ERR_CUDA and r.k == k, (warm, mode)
                 r.close()
     torch.cuda.synchronize()
+
+
+def count_launches(rt):
+    """Kernels launched one by one (not by a graph) in each of equal roll-outs, whose records are the same."""
+    fields = (W.WS_F_OBS, W.WS_F_ACTION, W.WS_F_LOGP, W.WS_F_REWARD, W.WS_F_DONE)
+    for env, path, h, kw in SHAPES:
+        r = W.Rollout(env, path, 300, 40, 15, h, h, **kw)
+        seen, records = [], set()
+        for _ in range(4):
+            r.reset(3)
+            rt.refuse_launch(-1)
+            r.rollout(10)
+            seen.append(rt.launches_seen())
+            records.add(b"".join(r.fetch(f, 0, 10).tobytes() for f in fields))
+        # launched directly once (no capture), captured (the launches are seen again), then through the graph
+        assert seen == [2, 2, 0, 0] and len(records) == 1, (env, path, seen)
+        r.reset(4)  # another seed: begins anew
+        rt.refuse_launch(-1)
+        r.rollout(10)
+        assert rt.launches_seen() == 2
+        r.close()
+
+
+def test_repeated_rollouts_go_through_a_graph(tmp_path):
+    need_gpu()
+    child("count_launches", tmp_path, module="test_gpu_short_rollouts")
