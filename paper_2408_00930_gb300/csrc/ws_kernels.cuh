@@ -110,11 +110,11 @@ struct TrainGroup {  // one policy and its critic, on slots [slot0, slot0 + n_sl
 };
 // Fused forward pass of a chunk (ws_train_fwd.cu): rows [q0, q0 + rows) of a group
 // from the ring through both networks (or the critic alone) into tb's activations,
-// outputs and values, with W2 packed by launch_train_pack.
+// outputs and values, with W2 packed by launch_train_pack (back: for the backward too).
 bool train_tc_supported(const PolicyShape &p);
 bool train_fwd_has_out(int out);
 size_t train_image_bytes(const PolicyShape &p);
-void launch_train_pack(const TrainGroup &g, uint8_t *img, cudaStream_t st);
+void launch_train_pack(const TrainGroup &g, uint8_t *img, bool back, cudaStream_t st);
 cudaError_t launch_train_fwd(const Dev &d, const TrainGroup &g, const TrainBufs &tb, uint64_t q0,
                              uint32_t n, uint32_t rows, int critic_only, cudaStream_t st);
 // Fused backward of the same chunk (ws_train_bwd.cu): dout (tb.out, tb.vout) through

@@ -986,7 +986,7 @@ void run_update(const Dev &d, const TrainBufs &tb, const TrainGroup *groups, int
     cudaMemsetAsync(tb.grad, 0, (na + nc) * 4, st);
     const double inv_r = 1.0 / (double)R;
     const size_t CH = chunk_rows(d, G.pol);
-    if (use_train_tc(d, G.pol)) launch_train_pack(G, tb.image, st);
+    if (use_train_tc(d, G.pol)) launch_train_pack(G, tb.image, true, st);
     for (size_t q0 = 0; q0 < R; q0 += CH) {
       const int rows = (int)((R - q0) < CH ? (R - q0) : CH);
       const bool fused = chunk_forward(d, tb, G, n, q0, rows, false, st);
@@ -1024,7 +1024,7 @@ void launch_advantages(const Dev &d, const TrainBufs &tb, const TrainGroup *grou
     const TrainGroup &G = groups[gi];
     const size_t R = (size_t)n * G.n_slots, CH = chunk_rows(d, G.pol);
     const bool both = d.env == WS_ENV_LANDSCAPE;  // its actor rebuilds the samples
-    if (use_train_tc(d, G.pol)) launch_train_pack(G, tb.image, st);
+    if (use_train_tc(d, G.pol)) launch_train_pack(G, tb.image, false, st);
     for (size_t q0 = 0; q0 < R; q0 += CH) {
       const int rows = (int)((R - q0) < CH ? (R - q0) : CH);
       chunk_forward(d, tb, G, n, q0, rows, !both, st);

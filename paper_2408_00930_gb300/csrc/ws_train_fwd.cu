@@ -319,11 +319,11 @@ cudaError_t run_fwd_h(const Dev &d, const Rows &rw, int in, int out, const Nets 
 }
 
 template <int H>
-void pack(const TrainGroup &g, uint8_t *img, cudaStream_t st) {
+void pack(const TrainGroup &g, uint8_t *img, bool back, cudaStream_t st) {
   const size_t o = g.pol.layer_offset(1), b = Geo<H>::IMAGE;
   const dim3 grid((H * H + 1023) / 1024, 2);
   k_pack_w2<H><<<grid, 256, 0, st>>>(g.params + o, g.critic + o, img, b, 0);
-  k_pack_w2<H><<<grid, 256, 0, st>>>(g.params + o, g.critic + o, img + 2 * b, b, 1);
+  if (back) k_pack_w2<H><<<grid, 256, 0, st>>>(g.params + o, g.critic + o, img + 2 * b, b, 1);
 }
 
 }  // namespace
@@ -341,10 +341,10 @@ size_t train_image_bytes(const PolicyShape &p) {
   return train_tc_supported(p) ? (size_t)4 * 4 * p.w[1] * p.w[1] : 0;
 }
 
-void launch_train_pack(const TrainGroup &g, uint8_t *img, cudaStream_t st) {
-  if (g.pol.w[1] == 64) pack<64>(g, img, st);
-  else if (g.pol.w[1] == 128) pack<128>(g, img, st);
-  else pack<256>(g, img, st);
+void launch_train_pack(const TrainGroup &g, uint8_t *img, bool back, cudaStream_t st) {
+  if (g.pol.w[1] == 64) pack<64>(g, img, back, st);
+  else if (g.pol.w[1] == 128) pack<128>(g, img, back, st);
+  else pack<256>(g, img, back, st);
 }
 
 // which: 0 both networks, 1 the critic alone.

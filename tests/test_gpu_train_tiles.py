@@ -4,6 +4,8 @@ import numpy as np
 import pytest
 
 from paper_2408_00930_gb300 import warpsci as W
+from tests.gpu_common import need_gpu
+from tests.refuse_launch import child
 
 pytestmark = pytest.mark.gpu
 LR = 1.0
@@ -65,3 +67,18 @@ def test_infinite_weight_and_a_partial_tile(algo, env, h, n, T, dim):
     def change(p):
         p[5] = np.inf
     _compare(algo, env, h, n, T, dim, change=change)
+
+
+def advantage_launches(rt):
+    r = W.Rollout(W.WS_ENV_CONTROL, W.WS_PATH_BATCHED_FP32, 100, 4, 9, 256, 256, flags=W.WS_FLAG_TRAIN)
+    r.reset(1)
+    r.rollout(4)
+    rt.refuse_launch(-1)
+    r.advantages(4)
+    assert rt.launches_seen() == 4  # returns, the forward's weight image, the forward, the store
+    r.close()
+
+
+def test_advantages_pack_for_the_forward_alone(tmp_path):
+    need_gpu()
+    child("advantage_launches", tmp_path, module="test_gpu_train_tiles")
