@@ -82,3 +82,13 @@ def advantage_launches(rt):
 def test_advantages_pack_for_the_forward_alone(tmp_path):
     need_gpu()
     child("advantage_launches", tmp_path, module="test_gpu_train_tiles")
+
+
+@pytest.mark.parametrize("algo,env,h,n,T,dim", [
+    ("ppo", W.WS_ENV_LANDSCAPE, 256, 8191, 9, 24), ("a2c", W.WS_ENV_LANDSCAPE, 256, 8191, 9, 16),
+    ("ppo", W.WS_ENV_LANDSCAPE, 64, 8191, 9, 10), ("a2c", W.WS_ENV_ECONOMY, 256, 150, 4, 0)])
+def test_many_tiles_without_an_output_layer(algo, env, h, n, T, dim):
+    # several tiles of each network per CTA, two chunks with a partial last tile, where the output layer, or its
+    # gradients, are formed outside the fused kernels (and at 256 units dW1 is summed in global memory)
+    agents = np.random.default_rng(2).integers(100, 200, n) if env == W.WS_ENV_ECONOMY else None
+    _compare(algo, env, h, n, T, dim, agents)
