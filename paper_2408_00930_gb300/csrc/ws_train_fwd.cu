@@ -293,7 +293,8 @@ template <int H, int OUT, int XV>
 cudaError_t run_fwd_x(const Dev &d, const Rows &rw, int in, const Nets &nets, cudaStream_t st) {
   const int xp = (in + 3) & ~3, out = OUT > 1 ? OUT : 1, smem = FwdSmem<H>::bytes(in, xp, out);
   const int off_w = FwdSmem<H>::w_fits(in, xp, out) ? FwdSmem<H>::off_w(xp) : 0;
-  cudaError_t e = set_smem_limit(k_train_fwd<H, OUT, XV>, smem);
+  // (one limit for every input width: another thread's launch may come between these two)
+  cudaError_t e = set_smem_limit(k_train_fwd<H, OUT, XV>, kSmemPerCta);
   if (e != cudaSuccess) return e;
   const int tiles = nets.count * (int)((rw.rows + kRows - 1) / kRows), ctas = 2 * sm_count();
   return launch_kernel(k_train_fwd<H, OUT, XV>, dim3(tiles < ctas ? tiles : ctas), dim3(kThreads), smem, st, d,

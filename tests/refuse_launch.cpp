@@ -1,10 +1,14 @@
 // Kernel launches that the runtime refuses, on call: loaded with its symbols global ahead of a library, this takes
 // the place of the runtime's two launch entries and passes every launch on, the chosen one with more shared memory
-// than any GPU has, so that the runtime turns it down (nothing reaches the GPU) and leaves its error as ever.
+// than any GPU has, so that the runtime turns it down (nothing reaches the GPU) and leaves its error as ever.  It
+// also counts the shared-memory limits that were set to another value than before.
 #include <cuda_runtime_api.h>
 #include <dlfcn.h>
 
-static int countdown = -1, seen = 0;
+#include <map>
+
+static int countdown = -1, seen = 0, changed = 0;
+static std::map<const void *, int> limits;
 
 static size_t smem_of(size_t asked) {
   ++seen;
@@ -23,6 +27,17 @@ void refuse_launch(int n) {
   seen = 0;
 }
 int launches_seen() { return seen; }
+int limits_changed() { return changed; }
+
+cudaError_t cudaFuncSetAttribute(const void *k, cudaFuncAttribute what, int value) {
+  static auto f = (cudaError_t(*)(const void *, cudaFuncAttribute, int))real("cudaFuncSetAttribute");
+  if (what == cudaFuncAttributeMaxDynamicSharedMemorySize) {
+    const auto it = limits.emplace(k, value).first;
+    changed += it->second != value;
+    it->second = value;
+  }
+  return f(k, what, value);
+}
 
 cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 grid, dim3 block, void **args, size_t smem, cudaStream_t st) {
   static auto f = (cudaError_t(*)(cudaKernel_t, dim3, dim3, void **, size_t, cudaStream_t))real("__cudaLaunchKernel");
