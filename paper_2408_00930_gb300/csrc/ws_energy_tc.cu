@@ -301,14 +301,10 @@ void launch_energy_tc_pack(const Dev &d, void *buf, cudaStream_t st) {
                                          img, tab);
 }
 
-void energy_tc_init(int M) {
-  int Mp, pc = 0;
-  for (int c = 1; c <= kMaxTcChunks; c *= 2) {
-    if (!energy_tc_chunks_ok(M, c)) continue;
-    energy_tc_shape(M, c, &Mp, &pc);
-    break;  // the smallest supported count has the largest chunk
-  }
-  cudaFuncSetAttribute(k_energy_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_for(pc));
+// One limit for every Gaussian count (a context of few Gaussians would else lower it for
+// the others).
+void energy_tc_init() {
+  cudaFuncSetAttribute(k_energy_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
 }
 
 void launch_energy_tc(const Dev &d, const void *buf, uint32_t off, int mode, cudaStream_t st) {

@@ -230,7 +230,7 @@ size_t energy_tc_bytes(int D, int M);
 bool energy_tc_supported(int D, int M);
 void launch_energy_tc_pack(const Dev &d, void *buf, cudaStream_t st);
 void launch_energy_tc(const Dev &d, const void *buf, uint32_t off, int mode, cudaStream_t st);
-void energy_tc_init(int M);
+void energy_tc_init();
 bool energy_tc_chunks_ok(int M, int chunks);
 
 // Y[M][N] = act(X W + b) with the plain path's FP32 dense kernel (X row-major

@@ -882,7 +882,7 @@ ws_status ws_create(const ws_config *cfg, void *state_buf, size_t state_bytes, v
   if (use_tc_control(cfg)) c->tc_grid = control_tc_default_grid(c->d);
   if (use_tc_layers(cfg)) dense_tc_init();
   if (c->d.mlp3) mlp3_tc_init();
-  if (use_tc_layers(cfg) && cfg->env == WS_ENV_LANDSCAPE) energy_tc_init((int)cfg->n_gauss);
+  if (use_tc_layers(cfg) && cfg->env == WS_ENV_LANDSCAPE) energy_tc_init();
   if (c->L.land_fused) land_tc_init();
   s = after_params_changed(c);
   if (s == WS_OK) s = ws_reset(c, cfg->param_seed);

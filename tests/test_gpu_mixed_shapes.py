@@ -56,3 +56,17 @@ def test_updates_in_threads():
         t.join()
     for a, b in zip(ref, got):
         assert b is not None and np.array_equal(a, b)
+
+
+def test_landscapes_of_different_sizes():
+    # a small BF16 landscape created after a large one
+    need_gpu()
+    make = lambda m: W.Rollout(W.WS_ENV_LANDSCAPE, W.WS_PATH_BATCHED_BF16, 200, 4, 3, 256, 256, dim=24, n_gauss=m)  # noqa: E731
+    large = make(4096)
+    want = large.fetch_raw(W.WS_F_STATE, 200 * (24 + 2) * 4)
+    small = make(64)
+    large.reset(large.cfg.param_seed)
+    large.sync()
+    assert np.array_equal(large.fetch_raw(W.WS_F_STATE, 200 * (24 + 2) * 4), want)
+    small.close()
+    large.close()
