@@ -604,6 +604,11 @@ ws_status enqueue_steps(ws_ctx *c, uint32_t n, cudaStream_t st) {
   return cuda_check(c, cudaGetLastError(), "step launch");
 }
 
+// The FP32 control path has a graph per roll-out length (its per-step graphs were one per
+// chunk and remainder): this many at most, then it begins anew.  1,000 lengths held 176 MB
+// on the host and 162 MB on the device; a capture is some 25 us of a roll-out of 60 up.
+constexpr size_t kF32Graphs = 64;
+
 // A caller's capture takes no roll-out: the steps would be counted (ws_get_step, ws_fetch)
 // without having run.  The graph launch of ws_rollout is refused by the runtime there.
 bool capturing(cudaStream_t st) {
@@ -619,6 +624,7 @@ ws_status graph_for(ws_ctx *c, uint32_t n, cudaGraphExec_t *out) {
     *out = it->second;
     return WS_OK;
   }
+  if (fused_f32_control(c) && c->graphs.size() >= kF32Graphs) drop_graphs(c);
   cudaError_t e = cudaStreamBeginCapture(c->capture, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) return cuda_check(c, e, "begin capture");
   ws_status s = enqueue_steps(c, n, c->capture);

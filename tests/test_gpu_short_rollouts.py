@@ -66,3 +66,27 @@ def count_launches(rt):
 def test_repeated_rollouts_go_through_a_graph(tmp_path):
     need_gpu()
     child("count_launches", tmp_path, module="test_gpu_short_rollouts")
+
+
+def many_lengths(rt):
+    r = W.Rollout(W.WS_ENV_CONTROL, W.WS_PATH_BATCHED_FP32, 9, 40, 15, 64, 64, chunk_steps=5)
+    r.reset(3)
+    for n in range(6, 106):
+        r.rollout(n)
+    r.sync()
+    rt.refuse_launch(-1)
+    r.rollout(105)
+    assert rt.launches_seen() == 0  # a late one: still there
+    r.rollout(6)
+    assert rt.launches_seen() == 3  # an early one: captured again (two chunks and the step count)
+    r.sync()
+    ref = W.Rollout(W.WS_ENV_CONTROL, W.WS_PATH_PLAIN_FP32, 9, 40, 15, 64, 64)
+    ref.reset(3)
+    ref.rollout(r.k)
+    for f in (W.WS_F_OBS, W.WS_F_ACTION, W.WS_F_LOGP):
+        assert r.fetch(f, r.k - 40, 40).tobytes() == ref.fetch(f, r.k - 40, 40).tobytes()
+
+
+def test_graphs_of_many_lengths_are_bounded(tmp_path):
+    need_gpu()
+    child("many_lengths", tmp_path, module="test_gpu_short_rollouts")
