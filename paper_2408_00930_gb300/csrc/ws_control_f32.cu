@@ -16,8 +16,8 @@
 //
 // What bounds it: the FP32 FMA pipe for many envs (131,072 envs, 4-256-256-2: 372
 // us per step against 1,003 us for the six kernels; 67% of the pipe's cycles busy
-// with the products' and tanhf's FMAs, floor 253 us), the step's own chain of
-// dependent phases for few (1,000 envs, 4-64-64-2: 1.2 us per step against 32 us).
+// with the products' and tanhf's FMAs, floor 253 us; at 255 registers the 64-row tile
+// spills 32 bytes), the step's own chain of dependent phases for few (1,000 envs, 4-64-64-2: 1.2 us per step against 32 us).
 #include <math.h>
 
 #include "ws_acrobot.cuh"
@@ -170,7 +170,7 @@ struct Cfg {
   static constexpr int S_H = S_X + kOP * RM;               // [NPAD][RM] h1 (then h2 in place)
   static constexpr int S_H2 = kSmall ? S_H + NPAD * RM : S_H;
   static constexpr int S_W1 = S_H2 + NPAD * RM;            // [kOP][NPAD]
-  static constexpr int S_W2 = S_W1 + kOP * NPAD;           // resident W2, or two stages
+  static constexpr int S_W2 = S_W1 + kOP * NPAD;           // resident W2, or ST stages
   static constexpr int S_W3 = S_W2 + (ST == 0 ? NPAD * NPAD : ST * f32::kKC * NPAD);  // [NPAD][NA]
   static constexpr int S_LG = S_W3 + NPAD * E::NA + 4;     // [NA][RM] logits
   static constexpr int S_RN = S_LG + E::NA * RM;           // [7][RM] uniform, reset words, sin, cos

@@ -36,6 +36,9 @@ constexpr int kFPart = kFTileM / kFG;
 // loads of 16 bytes and nothing is predicated.  Bound by the FP32 pipe: 3 D operations
 // and ~12 more per pair; 32,768 rows, D 24, 4,096 Gaussians: 526 us (floor 290 us);
 // with scalar, predicated loads, one thread per row and exposed tile loads 894 us.
+// (Registers are held to two blocks per SM up to D 24: 128, with 64 bytes spilled.  D over
+// 32 spills 476 at 255 registers: 4,096 rows, D 40 and 64, 1,000 Gaussians: 207 and 211 us,
+// one thread per row 490 and 501.)
 template <int DM>
 __global__ __launch_bounds__(kFT, DM <= 24 ? 2 : 1) void k_force_f32(Dev d, uint32_t n) {
   __shared__ __align__(16) float cs[kFTileM * DM];      // centres (then the groups' sums)

@@ -63,7 +63,7 @@ constexpr int kEBBytes = kEB * kKE * 2;       // two consecutive image blocks
 constexpr int kNS = 2;                        // shared-memory sweep-block buffers
 constexpr int kNT = 3;                        // TMEM accumulators of the sweep (128 columns each)
 constexpr int kHdr = 256;                     // energy image header: {blocks, positive blocks}
-constexpr int kEpi = 256, kThreads = kEpi + 64;  // + a loader warp and an MMA warp
+constexpr int kEpi = 256;                     // epilogue threads of both kernels
 // The roll-out kernel issues its sweep MMAs from two warps that take the even
 // and the odd blocks, so that one warp's waits run while the other's MMAs
 // keep the tensor core busy.
@@ -954,11 +954,12 @@ __global__ void __launch_bounds__(kRollThreads, 1)
 // accumulators of 2 x 32 columns per row.  The sign and 1 / w^2 ride in the force
 // image, so the epilogue is the exponential and the split alone.
 //
-// Bound by the tensor pipe's instructions: 21 per 128 Gaussians here.  Over 64-Gaussian
-// blocks with P through shared memory it was 34 (at ~115 cycles each, every one
-// reading 4 KB of A from shared memory): 1.436 ms for 8,192 envs x 50 steps x 4,096
-// Gaussians, D 24; now 0.70 ms (0.92 with one warp issuing both
-// products, 0.86 with the halves on alternate blocks).  The epilogue's ex2 floor is 0.17 ms.
+// 8,192 envs x 50 steps x 4,096 Gaussians, D 24: 0.70 ms, of which the ex2 alone take
+// 0.17.  Bound by the epilogue's tensor-memory round trips: two warps per scheduler, each
+// a chain of load, exponential, split and store (tensor pipe 25%, SFU 18%, issue slots
+// 26% busy, long scoreboard stalls).  The steps to it: 64-Gaussian blocks with P through
+// shared memory, 34 MMA instructions per 128 Gaussians instead of 21, 1.436 ms; P in tensor
+// memory 0.92; the halves on alternate blocks 0.86; two issuing warps 0.70.
 constexpr int kForceThreads = kEpi + 96;         // + a loader warp and two MMA warps
 constexpr int kFN = 32;                          // force columns: D coordinates, the sum, zeros
 constexpr int kFImgBytes = kFN * kBlk * 2;       // one plane of a block's force image

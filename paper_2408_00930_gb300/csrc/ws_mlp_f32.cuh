@@ -26,22 +26,6 @@ namespace f32 {
 
 constexpr int kKC = 16;  // weight rows per stage of a streamed layer
 
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-__device__ __forceinline__ uint64_t pair(float lo, float hi) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ float2 unpair(uint64_t v) {
-  float2 r;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-  return r;
-}
-
 // Asynchronous copy of BYTES (4 or 16) into shared memory, zeros if !valid.
 template <int BYTES>
 __device__ __forceinline__ void cp_async(void *dst, const void *src, bool valid) {
@@ -142,9 +126,9 @@ __device__ __forceinline__ void mma_rows(const float *__restrict__ A, const floa
       }
 #pragma unroll
       for (int i = 0; i < TM; ++i) {
-        const uint64_t aa = pair(a[i], a[i]);
+        const uint64_t aa = f2_pack(a[i], a[i]);
 #pragma unroll
-        for (int j = 0; j < CPT / 2; ++j) acc[i][j] = fma2(aa, b[j], acc[i][j]);
+        for (int j = 0; j < CPT / 2; ++j) acc[i][j] = f2_fma(aa, b[j], acc[i][j]);
       }
     }
   }
@@ -208,7 +192,7 @@ __device__ __forceinline__ void layer_tanh(float *H, const float *__restrict__ b
       float z[TM];
 #pragma unroll
       for (int i = 0; i < TM; ++i) {
-        const float2 p = unpair(acc[i][2 * q + (j >> 1)]);
+        const float2 p = f2_unpack(acc[i][2 * q + (j >> 1)]);
         z[i] = ((j & 1) ? p.y : p.x) + bc;
         if (kSmall) z[i] = tanhf(z[i]);
       }

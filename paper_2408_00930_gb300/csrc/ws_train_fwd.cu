@@ -291,6 +291,7 @@ int sm_count() {
 
 template <int H, int OUT, int XV>
 cudaError_t run_fwd_x(const Dev &d, const Rows &rw, int in, const Nets &nets, cudaStream_t st) {
+  if (in > XV * kXT) return cudaErrorInvalidValue;
   const int xp = (in + 3) & ~3, out = OUT > 1 ? OUT : 1, smem = FwdSmem<H>::bytes(in, xp, out);
   const int off_w = FwdSmem<H>::w_fits(in, xp, out) ? FwdSmem<H>::off_w(xp) : 0;
   // (one limit for every input width: another thread's launch may come between these two)
@@ -307,14 +308,17 @@ cudaError_t run_fwd(const Dev &d, const Rows &rw, int in, const Nets &nets, cuda
   return run_fwd_x<H, OUT, 12>(d, rw, in, nets, st);
 }
 
+// The input widths that occur with each output width of the envs' policies: 2 outputs
+// with 1 or 4 inputs (landscape, control), 3 with 6 (acrobot), 10 and 20 with 5, 10 or 16
+// (landscape, economy); any with the critic and with the output layer left out.
 template <int H>
 cudaError_t run_fwd_h(const Dev &d, const Rows &rw, int in, int out, const Nets &nets, cudaStream_t st) {
   switch (out) {
     case 1: return run_fwd<H, 1>(d, rw, in, nets, st);
-    case 2: return run_fwd<H, 2>(d, rw, in, nets, st);
-    case 3: return run_fwd<H, 3>(d, rw, in, nets, st);
-    case 10: return run_fwd<H, 10>(d, rw, in, nets, st);
-    case 20: return run_fwd<H, 20>(d, rw, in, nets, st);
+    case 2: return run_fwd_x<H, 2, 2>(d, rw, in, nets, st);
+    case 3: return run_fwd_x<H, 3, 8>(d, rw, in, nets, st);
+    case 10: return run_fwd_x<H, 10, 8>(d, rw, in, nets, st);
+    case 20: return run_fwd_x<H, 20, 8>(d, rw, in, nets, st);
     default: return run_fwd<H, 0>(d, rw, in, nets, st);
   }
 }
@@ -348,7 +352,7 @@ void launch_train_pack(const TrainGroup &g, uint8_t *img, bool back, cudaStream_
   else pack<256>(g, img, back, st);
 }
 
-// which: 0 both networks, 1 the critic alone.
+// Both networks of a group, or the critic alone.
 cudaError_t launch_train_fwd(const Dev &d, const TrainGroup &g, const TrainBufs &tb, uint64_t q0,
                              uint32_t n, uint32_t rows, int critic_only, cudaStream_t st) {
   const PolicyShape &p = g.pol;
