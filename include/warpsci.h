@@ -229,7 +229,9 @@ ws_status ws_step(ws_ctx *ctx);
 
 /* n_steps steps, asynchronous.  The batched paths launch cached CUDA graphs
  * (and the persistent fused kernel); the plain path launches every kernel of
- * every step from the host.  k advances by n_steps. */
+ * every step from the host.  k advances by n_steps.  A batched roll-out is
+ * refused (WS_ERR_CUDA) on a stream that is being captured: its steps would be
+ * counted without having run. */
 ws_status ws_rollout(ws_ctx *ctx, uint32_t n_steps);
 
 /* Discounted returns over the last n_steps ring rows (steps k-n..k-1):

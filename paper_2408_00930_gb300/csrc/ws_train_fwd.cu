@@ -10,8 +10,9 @@
 // written; the output layer in FP32 FMAs.  The parts ran as a gather, a thin GEMM,
 // a 128 x 128-tile GEMM that read h1 twice, and a thin output layer (65,536 rows x
 // 4-256-256-2: 20 + 63 + 17 us per network with a 64 MB activation read between each);
-// here 58,368 rows of both networks take 87 us, bound by the issue slots and the SFU
-// (60 M tanhf of two SFU results each).
+// here 58,368 rows of both networks take 87 us: issue slots 53% busy, the 60 M tanhf (two
+// SFU results each, 7.3 per clock per SM measured) 27 us, tensor pipe 21%; the rest are
+// the phases' loads and tails (long scoreboard) that the second CTA does not cover.
 #include <math.h>
 
 #include "ws_train_tc.cuh"
