@@ -154,29 +154,22 @@ __global__ __launch_bounds__(kFT, DM <= 24 ? 2 : 1) void k_force_f32(Dev d, uint
 }
 
 template <int DM>
-void launch_f32(const Dev &d, uint32_t n, cudaStream_t st) {
+cudaError_t launch_f32(const Dev &d, uint32_t n, cudaStream_t st) {
   const size_t rows = (size_t)n * d.n_envs;
-  k_force_f32<DM><<<(unsigned)((rows + kFRows - 1) / kFRows), kFT, 0, st>>>(d, n);
+  return launch_kernel(k_force_f32<DM>, dim3((unsigned)((rows + kFRows - 1) / kFRows)), dim3(kFT), 0, st, d, n);
 }
 
 }  // namespace
 
-void launch_forces(const Dev &d, uint32_t n_steps, cudaStream_t st) {
-  if (n_steps == 0) return;
-  if (d.fimg) {  // BF16 path with the fused kernel's energy image: tensor cores
-    launch_force_tc(d, d.limg, d.fimg, n_steps, st);
-    return;
-  }
-  if (d.dim <= 8)
-    launch_f32<8>(d, n_steps, st);
-  else if (d.dim <= 16)
-    launch_f32<16>(d, n_steps, st);
-  else if (d.dim <= 24)
-    launch_f32<24>(d, n_steps, st);
-  else if (d.dim <= 32)
-    launch_f32<32>(d, n_steps, st);
-  else
-    launch_f32<64>(d, n_steps, st);
+cudaError_t launch_forces(const Dev &d, uint32_t n_steps, cudaStream_t st) {
+  if (n_steps == 0) return cudaSuccess;
+  // BF16 path with the fused kernel's energy image: tensor cores
+  if (d.fimg) return launch_force_tc(d, d.limg, d.fimg, n_steps, st);
+  if (d.dim <= 8) return launch_f32<8>(d, n_steps, st);
+  if (d.dim <= 16) return launch_f32<16>(d, n_steps, st);
+  if (d.dim <= 24) return launch_f32<24>(d, n_steps, st);
+  if (d.dim <= 32) return launch_f32<32>(d, n_steps, st);
+  return launch_f32<64>(d, n_steps, st);
 }
 
 }  // namespace ws

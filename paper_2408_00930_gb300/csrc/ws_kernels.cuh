@@ -140,7 +140,7 @@ void launch_ppo_update(const Dev &d, const TrainBufs &tb, const TrainGroup *grou
                        uint32_t n, float lr, float eps, float c_v, float c_e, cudaStream_t st);
 
 // Landscape force -grad E(x') of the last n_steps ring rows (ws_force.cu).
-void launch_forces(const Dev &d, uint32_t n_steps, cudaStream_t st);
+cudaError_t launch_forces(const Dev &d, uint32_t n_steps, cudaStream_t st);
 
 // ---- BF16 tensor-core control path -----------------------------------------
 size_t control_tc_packed_bytes(const PolicyShape &shape);

@@ -1259,19 +1259,16 @@ __global__ void __launch_bounds__(kForceThreads, 1)
 template <int D>
 cudaError_t launch_force_d(const Dev &d, const uint8_t *eimg, const uint8_t *fimg, uint32_t n,
                            cudaStream_t st) {
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_force_tc<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, FSMEM);
-    attr = true;
-  }
+  const cudaError_t e = set_smem_limit(k_force_tc<D>, FSMEM);
+  if (e != cudaSuccess) return e;
   int dev = 0, sms = 148;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const size_t rows = (size_t)n * d.n_envs;
   const int n_tiles = (int)((rows + kRows - 1) / kRows);
   const int grid = n_tiles < sms ? n_tiles : sms;
-  k_force_tc<D><<<grid, kForceThreads, FSMEM, st>>>(d, eimg, eimg + land_blocks_off((int)d.n_gauss), fimg, n);
-  return cudaGetLastError();
+  return launch_kernel(k_force_tc<D>, dim3(grid), dim3(kForceThreads), FSMEM, st, d, eimg,
+                       eimg + land_blocks_off((int)d.n_gauss), fimg, n);
 }
 
 }  // namespace

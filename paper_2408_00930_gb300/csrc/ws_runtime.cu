@@ -1036,8 +1036,8 @@ ws_status ws_forces(ws_ctx *c, uint32_t n) {
   if (c->err != WS_OK) return c->err;
   if (!(c->cfg.flags & WS_FLAG_FORCE)) return WS_ERR_STATE;
   if (n == 0 || n > c->k_host || n > c->L.ring_steps) return WS_ERR_RANGE;
-  launch_forces(c->d, n, c->stream);
-  return cuda_check(c, cudaGetLastError(), "forces");
+  drop_earlier_error();
+  return cuda_check(c, launch_forces(c->d, n, c->stream), "forces");
 }
 
 }  // extern "C"

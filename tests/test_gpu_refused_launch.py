@@ -130,6 +130,24 @@ def refuse_rollouts(rt):
                     assert run(i)[1:] == (W.WS_ERR_CUDA, W.WS_ERR_CUDA), (path, env, i)
 
 
+def refuse_post_passes(rt):
+    """Every launch of the forces, the returns and a reset, on each path (BF16: the tensor-core force)."""
+    for path, h in ((W.WS_PATH_PLAIN_FP32, 64), (W.WS_PATH_BATCHED_FP32, 64), (W.WS_PATH_BATCHED_BF16, 256)):
+        for call in (lambda r: W.ws_forces(r.ctx, 2), lambda r: W.ws_returns(r.ctx, 2), lambda r: W.ws_reset(r.ctx, 7)):
+            def run(i):
+                r = context(W.WS_ENV_LANDSCAPE, h, 20, 4, 8, W.WS_FLAG_FORCE, path)
+                r.rollout(2)
+                rt.refuse_launch(i)
+                st, seen = call(r), rt.launches_seen()
+                rt.refuse_launch(-1)
+                r.close()
+                return seen, st
+            seen, st = run(-1)
+            assert st == W.WS_OK and seen > 0
+            for i in range(seen):
+                assert run(i)[1] == W.WS_ERR_CUDA, (path, i)
+
+
 def refuse_forward(rt):
     import torch
     x, w, y = (torch.zeros(4096, device="cuda") for _ in range(3))
@@ -146,7 +164,7 @@ def refuse_forward(rt):
         assert call(out) == W.WS_OK
 
 
-@pytest.mark.parametrize("what", ["refuse_rollouts", "refuse_forward"])
+@pytest.mark.parametrize("what", ["refuse_rollouts", "refuse_post_passes", "refuse_forward"])
 def test_calls_without_a_substitute(what, tmp_path):
     need_gpu()
     child(what, tmp_path, module="test_gpu_refused_launch")
