@@ -874,6 +874,13 @@ ws_status ws_create(const ws_config *cfg, void *state_buf, size_t state_bytes, v
       return r;
     }
   }
+  // kernel attributes before the first launch: setting one clears the thread's last error,
+  // and with it that of a refused launch
+  if (use_tc_control(cfg)) c->tc_grid = control_tc_default_grid(c->d);
+  if (use_tc_layers(cfg)) dense_tc_init();
+  if (c->d.mlp3) mlp3_tc_init();
+  if (use_tc_layers(cfg) && cfg->env == WS_ENV_LANDSCAPE) energy_tc_init();
+  if (c->L.land_fused) land_tc_init();
   launch_init_policy((float *)c->d.params, c->L.pol, cfg->param_seed, 0, c->stream);
   if (cfg->flags & WS_FLAG_TRAIN) {  // the critics: policy ids 2 (and 3, the planner's)
     launch_init_policy((float *)(c->state + c->L.critic_off), critic_shape(c->L.pol),
@@ -885,11 +892,6 @@ ws_status ws_create(const ws_config *cfg, void *state_buf, size_t state_bytes, v
   if (cfg->env == WS_ENV_ECONOMY)
     launch_init_policy((float *)c->d.params_planner, c->L.pol_planner, cfg->param_seed, 1, c->stream);
   if (cfg->env == WS_ENV_LANDSCAPE) launch_init_landscape(c->d, cfg->param_seed, c->stream);
-  if (use_tc_control(cfg)) c->tc_grid = control_tc_default_grid(c->d);
-  if (use_tc_layers(cfg)) dense_tc_init();
-  if (c->d.mlp3) mlp3_tc_init();
-  if (use_tc_layers(cfg) && cfg->env == WS_ENV_LANDSCAPE) energy_tc_init();
-  if (c->L.land_fused) land_tc_init();
   s = after_params_changed(c);
   if (s == WS_OK) s = ws_reset(c, cfg->param_seed);
   if (s == WS_OK) s = cuda_check(c, cudaStreamSynchronize(c->stream), "create sync");

@@ -148,6 +148,45 @@ def refuse_post_passes(rt):
                 assert run(i)[1] == W.WS_ERR_CUDA, (path, i)
 
 
+def refuse_creation(rt):
+    """Every launch of ws_create and of ws_load (parameters), on each path."""
+    shapes = [(W.WS_ENV_CONTROL, 64), (W.WS_ENV_ACROBOT, 64), (W.WS_ENV_ECONOMY, 128), (W.WS_ENV_ECONOMY, 64),
+              (W.WS_ENV_LANDSCAPE, 256), (W.WS_ENV_LANDSCAPE, 64)]
+    for path in (W.WS_PATH_PLAIN_FP32, W.WS_PATH_BATCHED_FP32, W.WS_PATH_BATCHED_BF16):
+        for env, h in shapes:
+            flags = W.WS_FLAG_TRAIN | (W.WS_FLAG_FORCE if env == W.WS_ENV_LANDSCAPE else 0)
+            kw = dict(dim=8, n_gauss=64) if env == W.WS_ENV_LANDSCAPE else {}
+
+            def create(i):
+                rt.refuse_launch(i)
+                try:
+                    r, st = W.Rollout(env, path, 5, 4, 9, h, h, flags=flags, **kw), W.WS_OK
+                except W.WarpSciError as e:
+                    r, st = None, e.status
+                seen = rt.launches_seen()
+                rt.refuse_launch(-1)
+                return r, st, seen
+            r, st, seen = create(-1)
+            assert st == W.WS_OK and seen > 0
+            n = sum(a * b + b for a, b in ((r.obs_dim(), h), (h, h), (h, r.n_out())))
+            n += sum(a * b + b for a, b in ((16, h), (h, h), (h, 10))) if env == W.WS_ENV_ECONOMY else 0
+            params = np.zeros(n, np.float32)
+
+            def load(r, i):
+                rt.refuse_launch(i)
+                st = W.ws_load(r.ctx, W.WS_F_PARAMS, params.ctypes.data, params.nbytes, 0, 2 ** 64 - 1)
+                got = st, rt.launches_seen()
+                rt.refuse_launch(-1)
+                r.close()
+                return got
+            for i in range(seen):
+                assert create(i)[:2] == (None, W.WS_ERR_CUDA), (path, env, h, i)
+            st, seen = load(r, -1)
+            assert st == W.WS_OK
+            for i in range(seen):
+                assert load(create(-1)[0], i)[0] == W.WS_ERR_CUDA, (path, env, h, i)
+
+
 def refuse_forward(rt):
     import torch
     x, w, y = (torch.zeros(4096, device="cuda") for _ in range(3))
@@ -164,7 +203,7 @@ def refuse_forward(rt):
         assert call(out) == W.WS_OK
 
 
-@pytest.mark.parametrize("what", ["refuse_rollouts", "refuse_post_passes", "refuse_forward"])
+@pytest.mark.parametrize("what", ["refuse_creation", "refuse_rollouts", "refuse_post_passes", "refuse_forward"])
 def test_calls_without_a_substitute(what, tmp_path):
     need_gpu()
     child(what, tmp_path, module="test_gpu_refused_launch")
