@@ -781,6 +781,50 @@ ws_status finish_update(ws_ctx *c, const TrainBufs &tb, uint32_t n, double *stat
 
 }  // namespace
 
+// ws_rollout; again: more roll-outs of this length may follow (a length that does not come
+// again is not captured).
+ws_status ws_rollout_some(ws_ctx *c, uint32_t n, bool again) {
+  if (!c) return WS_ERR_INVALID;
+  if (c->err != WS_OK) return c->err;
+  if (n == 0) return WS_OK;
+  drop_earlier_error();
+  ws_status s = WS_OK;
+  if (c->cfg.path == WS_PATH_PLAIN_FP32) {
+    for (uint32_t i = 0; i < n && s == WS_OK; ++i) s = enqueue_steps(c, 1, c->stream);
+  } else if (fused(c) || fused_f32_control(c)) {
+    // The first single chunk of a length under a seed and launch configuration is launched
+    // directly, without a capture (a new seed's step of one env: 37 us through a graph, 22
+    // directly); from the second on through a graph, whose launch is shorter (14.3 us
+    // against 17 directly; a served client of 1,000 envs and four chunks: 560 us against
+    // 615 with all four launched directly).  With more chunks the graph's shorter gaps
+    // count too (119 us against 123 launched one by one for a short roll-out).
+    if (n <= chunk_of(c) && !c->graphs.count(n) && !capturing(c->stream) &&
+        (c->ran_once.insert(n).second || !again)) {
+      s = enqueue_steps(c, n, c->stream);
+    } else {
+      cudaGraphExec_t g;
+      s = graph_for(c, n, &g);
+      if (s == WS_OK) s = cuda_check(c, cudaGraphLaunch(g, c->stream), "graph launch");
+    }
+  } else {
+    const uint32_t chunk = chunk_of(c);
+    const uint32_t full = n / chunk, rem = n % chunk;
+    cudaGraphExec_t g;
+    if (full) {
+      s = graph_for(c, chunk, &g);
+      for (uint32_t i = 0; i < full && s == WS_OK; ++i)
+        s = cuda_check(c, cudaGraphLaunch(g, c->stream), "graph launch");
+    }
+    if (rem && s == WS_OK) {
+      s = graph_for(c, rem, &g);
+      if (s == WS_OK) s = cuda_check(c, cudaGraphLaunch(g, c->stream), "graph launch");
+    }
+  }
+  c->ring_gen += 1;
+  if (s == WS_OK) c->k_host += n;
+  return s;
+}
+
 extern "C" {
 
 ws_status ws_query_bytes(const ws_config *cfg, size_t *state_bytes, size_t *ring_bytes,
@@ -932,46 +976,7 @@ ws_status ws_step(ws_ctx *c) {
   return s;
 }
 
-ws_status ws_rollout(ws_ctx *c, uint32_t n) {
-  if (!c) return WS_ERR_INVALID;
-  if (c->err != WS_OK) return c->err;
-  if (n == 0) return WS_OK;
-  drop_earlier_error();
-  ws_status s = WS_OK;
-  if (c->cfg.path == WS_PATH_PLAIN_FP32) {
-    for (uint32_t i = 0; i < n && s == WS_OK; ++i) s = enqueue_steps(c, 1, c->stream);
-  } else if (fused(c) || fused_f32_control(c)) {
-    // The first single chunk of a length under a seed and launch configuration is launched
-    // directly, without a capture (a new seed's step of one env: 37 us through a graph, 22
-    // directly); from the second on through a graph, whose launch is shorter (14.3 us
-    // against 17 directly; a served client of 1,000 envs and four chunks: 557 us against
-    // 626 with all four launched directly).  With more chunks the graph's shorter gaps
-    // count too (119 us against 123 launched one by one for a short roll-out).
-    if (n <= chunk_of(c) && !c->graphs.count(n) && !capturing(c->stream) && c->ran_once.insert(n).second) {
-      s = enqueue_steps(c, n, c->stream);
-    } else {
-      cudaGraphExec_t g;
-      s = graph_for(c, n, &g);
-      if (s == WS_OK) s = cuda_check(c, cudaGraphLaunch(g, c->stream), "graph launch");
-    }
-  } else {
-    const uint32_t chunk = chunk_of(c);
-    const uint32_t full = n / chunk, rem = n % chunk;
-    cudaGraphExec_t g;
-    if (full) {
-      s = graph_for(c, chunk, &g);
-      for (uint32_t i = 0; i < full && s == WS_OK; ++i)
-        s = cuda_check(c, cudaGraphLaunch(g, c->stream), "graph launch");
-    }
-    if (rem && s == WS_OK) {
-      s = graph_for(c, rem, &g);
-      if (s == WS_OK) s = cuda_check(c, cudaGraphLaunch(g, c->stream), "graph launch");
-    }
-  }
-  c->ring_gen += 1;
-  if (s == WS_OK) c->k_host += n;
-  return s;
-}
+ws_status ws_rollout(ws_ctx *c, uint32_t n) { return ws_rollout_some(c, n, true); }
 
 ws_status ws_returns(ws_ctx *c, uint32_t n) {
   if (!c) return WS_ERR_INVALID;

@@ -1,13 +1,13 @@
 // Kernel launches that the runtime refuses, on call: loaded with its symbols global ahead of a library, this takes
 // the place of the runtime's two launch entries and passes every launch on, the chosen one with more shared memory
 // than any GPU has, so that the runtime turns it down (nothing reaches the GPU) and leaves its error as ever.  It
-// also counts the shared-memory limits that were set to another value than before.
+// also counts the shared-memory limits that were set to another value than before, and the graphs made.
 #include <cuda_runtime_api.h>
 #include <dlfcn.h>
 
 #include <map>
 
-static int countdown = -1, seen = 0, changed = 0;
+static int countdown = -1, seen = 0, changed = 0, graphs = 0;
 static std::map<const void *, int> limits;
 
 static size_t smem_of(size_t asked) {
@@ -28,6 +28,13 @@ void refuse_launch(int n) {
 }
 int launches_seen() { return seen; }
 int limits_changed() { return changed; }
+int graphs_made() { return graphs; }
+
+cudaError_t cudaGraphInstantiate(cudaGraphExec_t *ex, cudaGraph_t g, unsigned long long flags) {
+  static auto f = (cudaError_t(*)(cudaGraphExec_t *, cudaGraph_t, unsigned long long))real("cudaGraphInstantiate");
+  ++graphs;
+  return f(ex, g, flags);
+}
 
 cudaError_t cudaFuncSetAttribute(const void *k, cudaFuncAttribute what, int value) {
   static auto f = (cudaError_t(*)(const void *, cudaFuncAttribute, int))real("cudaFuncSetAttribute");

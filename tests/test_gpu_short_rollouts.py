@@ -90,3 +90,24 @@ def many_lengths(rt):
 def test_graphs_of_many_lengths_are_bounded(tmp_path):
     need_gpu()
     child("many_lengths", tmp_path, module="test_gpu_short_rollouts")
+
+
+def served_graphs(rt):
+    srv = W.Server(256 << 20)
+    for path in (W.WS_PATH_BATCHED_FP32, W.WS_PATH_BATCHED_BF16):
+        for horizon, chunks, graphs in ((50, 1, 0), (130, 3, 0), (150, 3, 1), (230, 5, 1)):
+            before = rt.graphs_made()
+            q, _keep = W.make_request(W.WS_ENV_CONTROL, path, 300, horizon, 50, 60, 64, 64, seed=5)
+            st, rid = srv.submit(q)
+            assert st == W.WS_OK
+            for c in range(chunks):
+                assert srv.wait_chunk(rid, c, 30000) == W.WS_OK and srv.ack(rid, c) == W.WS_OK
+            assert rt.graphs_made() - before == graphs, (path, horizon)
+            assert srv.release(rid) == W.WS_OK
+    srv.close()
+
+
+def test_served_requests_capture_what_comes_again(tmp_path):
+    # three chunks of a length are the least for which a capture pays
+    need_gpu()
+    child("served_graphs", tmp_path, module="test_gpu_short_rollouts")
